@@ -41,10 +41,11 @@ extern "C" {
 
 #define AP_MIXED  0   /* FP32 pair/PME arithmetic, FP64 accumulation and PCG reductions */
 #define AP_FP64   1   /* FP64 everywhere (reference-grade, slow on GB300) */
-#define AP_FIXED  2   /* FP32 pair/PME arithmetic as AP_MIXED, but fields, forces, torque terms and
-                         the PME grid are accumulated in 64-bit fixed point (34 fractional bits;
-                         the energy 30), as the paper's fixed-point mode (Sec. 2.4): integer sums
-                         do not depend on the order of the additions, so every output is bitwise
+#define AP_FIXED  2   /* FP32 pair/PME arithmetic as AP_MIXED, but the PME grid and every sum that
+                         several threads add to in no fixed order are accumulated in 64-bit fixed
+                         point (34 fractional bits; the energy 30), as the paper's fixed-point mode
+                         (Sec. 2.4); the real-space sums of an atom are one thread group's, in a
+                         fixed order, and stored in fixed point. So every output is bitwise
                          reproducible from run to run and for any launch shape. Magnitudes must
                          stay below 2^29 in the units of the output (kcal/mol/A, e/A^2). */
 
@@ -310,10 +311,10 @@ int ap_lj_forces(ap_ctx *ctx, const double *d_lj, double *d_energy, double *d_fo
  * stream of its own; synchronizes. Errors through ap_last_error(NULL). */
 int ap_fp32_peak(int reps, double *h_tflops, int *h_sm_count);
 
-/* Diagnostics: erfc as the FP32 pair kernels evaluate it (the rational approximation of
- * Abramowitz & Stegun 7.1.26 times e^{-x^2} from the kernels' fast exponential) in d_approx,
- * and CUDA's erfcf in d_lib, for the n arguments d_x (x >= 0; device arrays of floats). Async
- * on `stream`; AP_ERR_ARG for a null pointer or n < 1. */
+/* Diagnostics: erfc as the FP32 pair kernels evaluate it (a polynomial of degree six in
+ * 1 / (1 + 0.4 x), the form of Abramowitz & Stegun 7.1.26 one degree higher, times e^{-x^2} from
+ * the kernels' fast exponential) in d_approx, and CUDA's erfcf in d_lib, for the n arguments d_x
+ * (x >= 0; device arrays of floats). Async on `stream`; AP_ERR_ARG for a null pointer or n < 1. */
 int ap_eval_erfc(const float *d_x, int n, float *d_approx, float *d_lib, void *stream);
 
 /* Batched replicas: many independent systems of uneven size advanced by one CUDA-graph

@@ -27,14 +27,13 @@ int dalloc(ap_ctx *ctx, P **p, size_t bytes) {
 }
 
 void free_all(ap_ctx *c) {
-    void *ptrs[] = {c->perm, c->iperm, c->bcenter, c->tiles, c->tshift, c->tshift_lo, c->tile_excl, c->excl_mask, c->cell_count,
-                    c->tmp_int, c->excl_off, c->excl_atoms, c->posq, c->dipd, c->quad0, c->quad1, c->alpha,
+    void *ptrs[] = {c->perm, c->iperm, c->bcenter, c->tiles, c->excl_mask, c->cell_count,
+                    c->tmp_int, c->posq, c->posw, c->dipd, c->quad0, c->quad1, c->alpha,
                     c->E, c->acc, c->rec, c->rot, c->mpl, c->frame_s, c->fvec, c->mu, c->r, c->qv, c->p, c->st,
                     c->grid, c->cgrid, c->cgrid_v, c->green, c->grid2, c->frc, c->gdip, c->gquad, c->red, c->mu_s, c->gbuf,
-                    c->tile_off, c->chunk_j, c->chunk_pos, c->chunk_src, c->chunk_mask, c->chunk_flag, c->nchunk,
-                    c->work, c->n_work, c->red_part, c->pmask, c->pmask_t, c->mlp_feat, c->mlp_y, c->smask, c->smask_t, c->pstart, c->sstart, c->e1s,
-                    c->dg, c->stb, c->stw, c->grid_fx, c->work_off,
-                    c->hist_count, c->item_start, c->scan_tmp, c->mu_f, c->r_f, c->q_f, c->dga_f};
+                    c->tile_off, c->ncand, c->cand_j, c->cand_pos, c->cand_mask, c->list, c->list_meta,
+                    c->red_part, c->mlp_feat, c->mlp_y, c->e1s, c->dg, c->stb, c->stw, c->grid_fx,
+                    c->hist_count, c->mu_f, c->r_f, c->q_f, c->dga_f, c->bhalf, c->nb_info};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     diis_release(c);
@@ -77,9 +76,10 @@ int create_impl(ap_ctx *ctx, const ap_params *P, void *stream) {
     if ((r = dalloc(ctx, &ctx->iperm, sizeof(int) * np))) return r;
     if ((r = dalloc(ctx, &ctx->bcenter, sizeof(float4) * nb))) return r;
     if ((r = dalloc(ctx, &ctx->tile_off, sizeof(int) * (nb + 1)))) return r;
-    if ((r = dalloc(ctx, &ctx->nchunk, sizeof(int) * nb))) return r;
-    if ((r = dalloc(ctx, &ctx->n_work, sizeof(int) * 4))) return r;
+    if ((r = dalloc(ctx, &ctx->bhalf, sizeof(float4) * nb))) return r;
+    if ((r = dalloc(ctx, &ctx->nb_info, sizeof(int) * 8))) return r;
     if ((r = dalloc(ctx, (char **)&ctx->posq, 4 * es * np))) return r;
+    if ((r = dalloc(ctx, (char **)&ctx->posw, 4 * es * np))) return r;
     if ((r = dalloc(ctx, &ctx->stb, sizeof(int4) * np))) return r;
     if ((r = dalloc(ctx, (char **)&ctx->stw, 4 * es * np))) return r;
     if ((r = dalloc(ctx, (char **)&ctx->dipd, 4 * es * np))) return r;
@@ -189,23 +189,27 @@ int permanent_field(ap_ctx *ctx, const double *d_xyz, const double *d_mpole, con
     int r = cfg_load(ctx, d_xyz, d_mpole, d_frame, d_alpha);
     if (r) return r;
     // the reciprocal branch needs only the loaded configuration. Run directly, it starts
-    // on the second stream while the list filter and the pair masks run here (one system
-    // leaves the GPU room for both); captured into a batch graph, where many replicas
-    // already fill the GPU, it starts after them (measured faster both ways)
+    // on the second stream while the pair lists are made here (one system leaves the GPU room
+    // for both); captured into a batch graph, where many replicas already fill the GPU, it
+    // starts after them, or in a batch of several replicas runs in the same chain (measured faster
+    // both ways)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     AP_CUDA(cudaStreamIsCapturing(ctx->s0, &cap));
     const bool early = cap == cudaStreamCaptureStatusNone;
-    if (!early && (r = filter_launch(ctx, ctx->s0))) return r;
-    AP_CUDA(cudaEventRecord(ctx->ev_fork, ctx->s0));
-    AP_CUDA(cudaStreamWaitEvent(ctx->s1, ctx->ev_fork, 0));
-    if ((r = pme_multipole_field(ctx, ctx->s1))) return r;
-    if (early && (r = filter_launch(ctx, ctx->s0))) return r;
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
+    const cudaStream_t aux = aux_stream(ctx, ctx->s0, ctx->s1);
+    if (!early && (r = lists_launch(ctx, ctx->s0))) return r;
+    if (aux != ctx->s0) {
+        AP_CUDA(cudaEventRecord(ctx->ev_fork, ctx->s0));
+        AP_CUDA(cudaStreamWaitEvent(aux, ctx->ev_fork, 0));
+    }
+    if ((r = pme_multipole_field(ctx, aux))) return r;
+    if (early && (r = lists_launch(ctx, ctx->s0))) return r;
     if ((r = real_field_launch(ctx, ctx->s0))) return r;
-    AP_CUDA(cudaEventRecord(ctx->ev_join, ctx->s1));
-    AP_CUDA(cudaStreamWaitEvent(ctx->s0, ctx->ev_join, 0));
+    if (aux != ctx->s0) {
+        AP_CUDA(cudaEventRecord(ctx->ev_join, aux));
+        AP_CUDA(cudaStreamWaitEvent(ctx->s0, ctx->ev_join, 0));
+    }
     if ((r = field_finish(ctx, d_field))) return r;
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
     ctx->config_valid = 1;
     return AP_OK;
 }
@@ -288,7 +292,7 @@ int dipole_field_matvec(ap_ctx *ctx, const double *d_v, double *d_out) {
 int ap_list_stats(const ap_ctx *ctx, int *h_blocks, int *h_tiles, int *h_excl_tiles) {
     if (!ctx) return AP_ERR_ARG;
     if (h_blocks) *h_blocks = ctx->n_blocks;
-    if (h_tiles) *h_tiles = ctx->n_tiles;
+    if (h_tiles) *h_tiles = (ctx->n_tiles + ctx->n_blocks) / 2;   // kept in both orders, diagonal ones once
     if (h_excl_tiles) *h_excl_tiles = ctx->n_excl_tiles;
     return AP_OK;
 }
@@ -327,7 +331,7 @@ int ap_time_kernel(ap_ctx *ctx, int which, int reps, double *h_ms) {
         case AP_KERNEL_SPREAD_MULTIPOLES: return pme_stage_launch(ctx, 3, st);
         case AP_KERNEL_PAIR_FORCES: return pair_forces_launch(ctx, st);
         case AP_KERNEL_PCG_VECTORS: return pcg_vectors_launch(ctx, st);
-        case AP_KERNEL_REAL_MATVEC2: return dp_matvec2_launch(ctx, st, 0);
+        case AP_KERNEL_REAL_MATVEC2: return dp_matvec2_launch(ctx, st);
         case AP_KERNEL_FFT_ROUNDTRIP: return pme_stage_launch(ctx, 4, st);
         case AP_KERNEL_PME_DIPOLES: return pme_dipole_field(ctx, ctx->p, st);
         case AP_KERNEL_DIPOLE_OPERATOR: return dipole_operator_into(ctx, st, ctx->s1);
@@ -381,17 +385,6 @@ int ap_time_kernel(ap_ctx *ctx, int which, int reps, double *h_ms) {
     if (gx) cudaGraphExecDestroy(gx);
     cudaEventDestroy(a);
     cudaEventDestroy(b);
-    // the timed launches accumulated into scratch buffers: clear them for the next call
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
-    if (which == AP_KERNEL_REAL_MATVEC2) {
-        const int rc = dp_matvec2_launch(ctx, ctx->s0, 1);
-        if (rc) return rc;
-    }
-    if (which == AP_KERNEL_PAIR_FORCES) {
-        AP_CUDA(cudaMemsetAsync(ctx->frc, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
-        AP_CUDA(cudaMemsetAsync(ctx->gdip, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
-        AP_CUDA(cudaMemsetAsync(ctx->gquad, 0, sizeof(double) * 6 * ctx->n_pad, ctx->s0));
-    }
     *h_ms = total / reps;
     return AP_OK;
 }

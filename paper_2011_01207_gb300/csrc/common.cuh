@@ -10,7 +10,12 @@
 #include "../../include/amoebapol.h"
 
 #define AP_WARP 32
-#define AP_BLOCK_ATOMS 32          // atoms per block (one warp lane each), paper Sec. 2.3: B_size = 32
+#define AP_BLOCK_ATOMS 32          // atoms per block, paper Sec. 2.3: B_size = 32
+#define AP_CHUNK 640               // candidate atoms of a block staged in shared memory at once
+#define AP_CAND_SELF (1 << 30)     // a candidate that is an atom of the block itself
+#define AP_LIST_PER_TILE 528       // capacity of the pair lists, entries per tile: 32 candidates x 16 target
+                                   // pairs, and the padding of a chunk's 16 lists spread over its tiles
+#define AP_LIST_PER_BLOCK 256
 
 // physical constants (readings: the paper gives none)
 #define AP_COULOMB 332.063713       // kcal A / (mol e^2)
@@ -62,6 +67,13 @@ __device__ __forceinline__ double acc_value(const double *acc, size_t k, int fix
     return fixed ? ap_from_fx(reinterpret_cast<const long long *>(acc)[k]) : acc[k];
 }
 
+// one block pair (I, J) in block I's list: J, its exclusion-mask slot or -1, and the origin of block J
+// relative to block I's, periodic image included (c_J - c_I + L k), as hi + lo float pairs
+struct __align__(16) TileRec {
+    int J, excl;
+    float hx, hy, hz, lx, ly, lz;
+};
+
 struct ap_ctx {
     ap_params prm;
     int prec = AP_MIXED;      // arithmetic: AP_MIXED (FP32 pairs/PME) or AP_FP64
@@ -73,56 +85,46 @@ struct ap_ctx {
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     std::string err;
     int sm_count = 0;
+    int one_stream = 0;                 // a batch of several replicas is being captured: every replica's
+                                        // kernels in one chain (ap_batch_capture)
 
     // neighbour blocks
     int *perm = nullptr;      // [n_pad] slot -> atom (-1 for padding)
     int *iperm = nullptr;     // [n] atom -> slot
     float4 *bcenter = nullptr;   // [n_blocks] block centre (x,y,z) at the last build
-    int2 *tiles = nullptr;       // [cap_tiles] block pairs (I <= J), sorted by I then J
-    float4 *tshift = nullptr;    // [cap_tiles] origin of block J relative to block I's, periodic image
-                                 // included (c_J - c_I + L k), as hi + lo float pairs with tshift_lo
-    float4 *tshift_lo = nullptr; // [cap_tiles]
-    int *tile_excl = nullptr;    // [cap_tiles] exclusion-mask slot or -1
-    unsigned *excl_mask = nullptr;  // [cap_excl][32]
+    TileRec *tiles = nullptr;    // [cap_tiles] block pairs (I, J), both orders, sorted by I then J
+    unsigned *excl_mask = nullptr;  // [cap_excl] words, 32 per slot: word j-lane, bit i-lane
     int n_tiles = 0, cap_tiles = 0, n_excl_tiles = 0, cap_excl = 0;
     int *tile_off = nullptr;     // [n_blocks+1] first tile of each block
-    int minimg = 1;              // per-pair minimum image (small boxes) vs per-tile shifts
-    // per-configuration filtered chunks (capacity cap_chunks = cap_tiles chunks of 32)
-    int *chunk_j = nullptr;      // [cap][32] j slot or -1
-    void *chunk_pos = nullptr;   // T4 [cap][32] j position (image next to block I) and Thole factor
-    int *chunk_src = nullptr;    // [cap][32] exclusion source (slot << 5 | j-lane) or -1
-    unsigned *chunk_mask = nullptr;  // [cap][32] exclusion bits (i-lane word, bit = chunk position)
-    int *chunk_flag = nullptr;   // [cap] 1 if the chunk holds excluded pairs
-    int *nchunk = nullptr;       // [n_blocks]
-    int2 *work = nullptr;        // [n_blocks + cap] (I, chunk) items, chunk -1 = diagonal block
-    int *work_off = nullptr;     // [n_blocks + 1] first item of each block
-    int *n_work = nullptr;       // device: [0] work items, [1] in-range pairs of the configuration
-    int *item_start = nullptr;   // [work + 1] exclusive prefix of the items' weights (pairs + staging cost)
-    int *scan_tmp = nullptr;     // chunk sums of that prefix
-    unsigned *pmask = nullptr;   // [work][32] in-range pair bits per item (i-lane word, bit = j-lane)
-    unsigned *pmask_t = nullptr; // [work][32] the transpose (j-lane word, bit = i-lane)
-    unsigned *smask = nullptr;   // [work][32] pairs closer than AP_SHORT_RANGE (learned-guess feature)
-    unsigned *smask_t = nullptr; // its transpose
-    unsigned *pstart = nullptr;  // [work][32] each lane's start in the item's pair sides (side_start)
-    unsigned *sstart = nullptr;  // the same for the short-range sides
+    int image_dims = 0;          // bit d: the box is too short along d for one image per tile
+    // pair lists of the configuration (lists.cu, walked as in pair_walk.cuh)
+    int list_mult = 1;           // images an atom can appear in beside one block (2 per short dimension)
+    int4 *ncand = nullptr;       // [n_blocks] candidate atoms in the block's four segments
+    int *cand_j = nullptr;       // [cap][32] candidate's slot | AP_CAND_SELF
+    void *cand_pos = nullptr;    // T4 [cap][32] candidate's position beside the block, Thole factor
+    uint4 *cand_mask = nullptr;  // [cap][32] in-range, short-range and exclusion bits (bit i-lane), cand_j
+    unsigned *list = nullptr;    // the lists' entries, two per word
+    uint2 *list_meta = nullptr;  // [chunk][16] where each target pair's list lies
     double *e1s = nullptr;       // [3][n_pad] short-range first-order induced field (feature)
-    int cap_chunks = 0;
+    long cap_lists = 0;          // tiles x images the candidate and list arrays hold
     int lists_valid = 0;
     // scratch for the build
     int *cell_count = nullptr; int cap_cells = 0;
     int *tmp_int = nullptr; int cap_tmp = 0;
-    int *excl_off = nullptr, *excl_atoms = nullptr; int cap_excl_atoms = 0;   // copy of the CSR
+    float4 *bhalf = nullptr;     // [n_blocks] half extents of the blocks at the last build
+    int *nb_info = nullptr;      // [8] a build's results read back together (neighbour.cu)
 
     // configuration (sorted slots; element type T = float or double). Positions are stored
     // relative to the origin of the slot's block (its centre at the list build, bcenter):
     // small numbers, so FP32 keeps ~1e-6 A at any box size; pair kernels see differences
     // only, and the chunk positions are formed relative to block I's origin in FP64.
     void *posq = nullptr;     // T4: x, y, z (relative to the block origin), q
+    void *posw = nullptr;     // T4: x, y, z again, alpha^-1/2 (Thole); padding far outside
     int4 *stb = nullptr;      // [n_pad] smooth-PME stencil origin floor(K x / L) mod K per dimension
     void *stw = nullptr;      // T4 [n_pad] its fractional part K x / L - floor(K x / L), from FP64
     void *dipd = nullptr;     // T4: dx, dy, dz, alpha^-1/2 (Thole)
     void *quad0 = nullptr;    // T4: Qxx, Qxy, Qxz, Qyy
-    void *quad1 = nullptr;    // T4: Qyz, Qzz, alpha, 0
+    void *quad1 = nullptr;    // T4: Qyz, Qzz, alpha, q
     double *alpha = nullptr;  // [n_pad]
     double *E = nullptr;      // [3][n_pad] permanent field (SoA)
     double *acc = nullptr;    // [3][n_pad] real-space accumulator
@@ -186,47 +188,6 @@ struct ap_ctx {
     int graph_tried = 0;
 };
 
-// arguments of the real-space kernels that iterate the filtered work items
-struct WorkArgs {
-    const int2 *work;
-    const int *n_work;
-    const int *chunk_j;
-    const void *chunk_pos;
-    const unsigned *chunk_mask;
-    const int *chunk_flag;
-    const int *tile_excl;      // for the diagonal block's own mask
-    const int *tile_off;
-    const unsigned *excl_mask;
-    const unsigned *pmask;
-    const unsigned *pmask_t;
-    const unsigned *smask;
-    const unsigned *smask_t;
-    const unsigned *pstart;    // per (item, lane): packed start of the lane's share of the sides
-    const unsigned *sstart;
-    const int *item_start;     // exclusive prefix of the item weights; [n_work] = total
-};
-
-inline WorkArgs work_args(const ap_ctx *ctx) {
-    WorkArgs w;
-    w.work = ctx->work;
-    w.n_work = ctx->n_work;
-    w.chunk_j = ctx->chunk_j;
-    w.chunk_pos = ctx->chunk_pos;
-    w.chunk_mask = ctx->chunk_mask;
-    w.chunk_flag = ctx->chunk_flag;
-    w.tile_excl = ctx->tile_excl;
-    w.tile_off = ctx->tile_off;
-    w.excl_mask = ctx->excl_mask;
-    w.pmask = ctx->pmask;
-    w.pmask_t = ctx->pmask_t;
-    w.smask = ctx->smask;
-    w.smask_t = ctx->smask_t;
-    w.pstart = ctx->pstart;
-    w.sstart = ctx->sstart;
-    w.item_start = ctx->item_start;
-    return w;
-}
-
 // error helpers -------------------------------------------------------------------------
 int ap_fail(ap_ctx *c, int code, const std::string &msg);
 #define AP_CUDA(call)                                                                    \
@@ -242,6 +203,9 @@ int ap_fail(ap_ctx *c, int code, const std::string &msg);
             return ap_fail(ctx, AP_ERR_CUDA, std::string(#call) + ": cufft error " + std::to_string((int)r_)); \
     } while (0)
 
+// the stream of the reciprocal branch beside `main`, whose usual partner is `aux`
+inline cudaStream_t aux_stream(const ap_ctx *ctx, cudaStream_t main, cudaStream_t aux) { return ctx->one_stream ? main : aux; }
+
 // launch helpers --------------------------------------------------------------------------
 static inline int ap_grid_for(long n, int threads) { return (int)((n + threads - 1) / threads); }
 
@@ -249,8 +213,8 @@ static inline int ap_grid_for(long n, int threads) { return (int)((n + threads -
 int nb_build(ap_ctx *ctx, const double *d_xyz, const int *d_off, const int *d_atoms, int n_excl);
 int cfg_load(ap_ctx *ctx, const double *d_xyz, const double *d_mpole, const int *d_frame,
              const double *d_alpha);
-int filter_launch(ap_ctx *ctx, cudaStream_t s);
-int filter_alloc(ap_ctx *ctx);
+int lists_launch(ap_ctx *ctx, cudaStream_t s);   // pair lists of the loaded configuration
+int lists_alloc(ap_ctx *ctx);
 int real_field_launch(ap_ctx *ctx, cudaStream_t s);
 int real_matvec_launch(ap_ctx *ctx, const void *p, cudaStream_t s);
 int real_matvec_resident_per_sm(ap_ctx *ctx);
@@ -301,6 +265,7 @@ int dp_solve(ap_ctx *ctx, const double *gd, const double *gp, double tol, int ma
 int dp_forces(ap_ctx *ctx, const double *d_mu_d, const double *d_mu_p, double *d_energy, double *d_forces,
               double *d_virial);
 int dp_info(ap_ctx *ctx, ap_solve_info *info);
-int dp_matvec2_launch(ap_ctx *ctx, cudaStream_t s, int clear);
+int dp_matvec2_launch(ap_ctx *ctx, cudaStream_t s);
 void dp_release(ap_ctx *ctx);
+void diis_forget_graph(ap_ctx *ctx);
 void dp_forget_graph(ap_ctx *ctx);   // drop the captured two-set solve loop (launch shapes changed)

@@ -68,7 +68,8 @@ __global__ void k_load(const double *__restrict__ xyz, const double *__restrict_
                        typename V4<T>::type *__restrict__ quad0, typename V4<T>::type *__restrict__ quad1,
                        double *__restrict__ alpha_s, double *__restrict__ rot, double *__restrict__ mpl,
                        int *__restrict__ frame_s, double *__restrict__ fvec, int *__restrict__ bad, int3 K,
-                       double3 sK, int4 *__restrict__ stb, typename V4<T>::type *__restrict__ stw) {
+                       double3 sK, int4 *__restrict__ stb, typename V4<T>::type *__restrict__ stw,
+                       typename V4<T>::type *__restrict__ posw) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int s = iperm[i];
@@ -109,6 +110,8 @@ __global__ void k_load(const double *__restrict__ xyz, const double *__restrict_
     T4 v;
     v.x = (T)(p[0] - cc[0]); v.y = (T)(p[1] - cc[1]); v.z = (T)(p[2] - cc[2]); v.w = (T)m[0];
     posq[s] = v;
+    v.w = (T)(al > 0.0 ? rsqrt(al) : 1e4);
+    posw[s] = v;
     // smooth-PME stencil from the FP64 position: u = K x / L, origin floor(u) mod K, fraction
     {
         const int Ks[3] = {K.x, K.y, K.z};
@@ -131,7 +134,7 @@ __global__ void k_load(const double *__restrict__ xyz, const double *__restrict_
     dipd[s] = v;
     v.x = (T)Qg[0][0]; v.y = (T)Qg[0][1]; v.z = (T)Qg[0][2]; v.w = (T)Qg[1][1];
     quad0[s] = v;
-    v.x = (T)Qg[1][2]; v.y = (T)Qg[2][2]; v.z = (T)al; v.w = (T)0;
+    v.x = (T)Qg[1][2]; v.y = (T)Qg[2][2]; v.z = (T)al; v.w = (T)m[0];
     quad1[s] = v;
     alpha_s[s] = al;
     for (int a = 0; a < 3; ++a)
@@ -142,10 +145,11 @@ __global__ void k_load(const double *__restrict__ xyz, const double *__restrict_
     frame_s[3 * s + 2] = (type != AP_FRAME_NONE && xa >= 0) ? iperm[xa] : -1;
 }
 
-// padding slots: NaN positions make every pair test false; zero multipoles and alpha
+// padding slots: NaN positions, or (posw) positions out of every range; zero multipoles and alpha
 template <class T>
 __global__ void k_pad(int n, int n_pad, typename V4<T>::type *posq, typename V4<T>::type *dipd,
-                      typename V4<T>::type *quad0, typename V4<T>::type *quad1, double *alpha_s, int *frame_s) {
+                      typename V4<T>::type *quad0, typename V4<T>::type *quad1, double *alpha_s, int *frame_s,
+                      typename V4<T>::type *posw) {
     int s = n + blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n_pad) return;
     typedef typename V4<T>::type T4;
@@ -155,6 +159,8 @@ __global__ void k_pad(int n, int n_pad, typename V4<T>::type *posq, typename V4<
     T4 pp = z;
     pp.x = pp.y = pp.z = nanv;
     posq[s] = pp;
+    pp.x = pp.y = pp.z = (T)1e17;
+    posw[s] = pp;
     dipd[s] = z;
     quad0[s] = z;
     quad1[s] = z;
@@ -202,10 +208,11 @@ int load_t(ap_ctx *ctx, const double *d_xyz, const double *d_mpole, const int *d
         d_xyz, d_mpole, d_frame, d_alpha, ctx->iperm, ctx->bcenter, ctx->n, L, iL, (T4 *)ctx->posq, (T4 *)ctx->dipd,
         (T4 *)ctx->quad0, (T4 *)ctx->quad1, ctx->alpha, ctx->rot, ctx->mpl, ctx->frame_s, ctx->fvec, bad,
         make_int3(ctx->K[0], ctx->K[1], ctx->K[2]),
-        make_double3(ctx->K[0] / P.box[0], ctx->K[1] / P.box[1], ctx->K[2] / P.box[2]), ctx->stb, (T4 *)ctx->stw);
+        make_double3(ctx->K[0] / P.box[0], ctx->K[1] / P.box[1], ctx->K[2] / P.box[2]), ctx->stb, (T4 *)ctx->stw,
+        (T4 *)ctx->posw);
     if (ctx->n_pad > ctx->n)
         k_pad<T><<<1, 32, 0, ctx->s0>>>(ctx->n, ctx->n_pad, (T4 *)ctx->posq, (T4 *)ctx->dipd, (T4 *)ctx->quad0,
-                                        (T4 *)ctx->quad1, ctx->alpha, ctx->frame_s);
+                                        (T4 *)ctx->quad1, ctx->alpha, ctx->frame_s, (T4 *)ctx->posw);
     AP_CUDA(cudaGetLastError());
     return AP_OK;
 }

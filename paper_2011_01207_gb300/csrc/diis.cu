@@ -147,10 +147,10 @@ __device__ bool bordered_solve(const DiisState *st, int j, int w, double *c) {
     return true;
 }
 
-// y = alpha (E + T x), e = y - x into ring position j; partial e . e_i for the window; clears
-// acc for the next operator application. The last block finishes the iteration.
+// y = alpha (E + T x), e = y - x into ring position j; partial e . e_i for the window. The
+// last block finishes the iteration.
 template <class T>
-__global__ void __launch_bounds__(NT) k_diis_step(const double *__restrict__ x, double *__restrict__ acc,
+__global__ void __launch_bounds__(NT) k_diis_step(const double *__restrict__ x, const double *__restrict__ acc,
                                                   const T *__restrict__ rec, const double *__restrict__ E,
                                                   const double *__restrict__ alpha, double self_coef, int n_pad,
                                                   int n, double *__restrict__ ys, double *__restrict__ es,
@@ -172,7 +172,6 @@ __global__ void __launch_bounds__(NT) k_diis_step(const double *__restrict__ x, 
             const double xv = x[k];
             const double y = a * (E[k] + acc_value(acc, k, fixed) + (double)rec[k] + self_coef * xv);
             const double e = y - xv;
-            acc[k] = 0.0;
             ys[j * stride + k] = y;
             es[j * stride + k] = e;
 #pragma unroll
@@ -398,7 +397,6 @@ int diis_t(ap_ctx *ctx, const double *d_guess, double tol, int max_iter, int dep
     const int nb = ap_grid_for(ctx->n_pad, NT);
     DiisState *st = (DiisState *)ctx->diis_st;
     k_diis_init<<<1, 32, 0, s>>>(st, tol, max_iter, depth);
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, s));
     k_diis_guess<T><<<nb, NT, 0, s>>>(d_guess, ctx->E, ctx->alpha, ctx->perm, ctx->n, ctx->n_pad, ctx->mu,
                                        (T4 *)ctx->p);
     AP_CUDA(cudaGetLastError());
@@ -445,6 +443,11 @@ int diis_solve(ap_ctx *ctx, const double *d_guess, double tol, int max_iter, int
                ap_solve_info *info) {
     return ctx->prec == AP_FP64 ? diis_t<double>(ctx, d_guess, tol, max_iter, depth, d_mu, info)
                                 : diis_t<float>(ctx, d_guess, tol, max_iter, depth, d_mu, info);
+}
+
+void diis_forget_graph(ap_ctx *ctx) {
+    if (ctx->diis_exec) cudaGraphExecDestroy(ctx->diis_exec);
+    ctx->diis_exec = nullptr;
 }
 
 void diis_release(ap_ctx *ctx) {

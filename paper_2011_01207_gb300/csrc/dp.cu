@@ -347,7 +347,7 @@ struct DpVecs {
     const void *rec[2];
 };
 
-// r_k = E_k - A mu_k; clears the accumulators and the directions; partial r.z and z.z of
+// r_k = E_k - A mu_k; clears the directions; partial r.z and z.z of
 // both systems. The last block sets the initial state.
 template <class T>
 __global__ void k_dp_init_residual(const double *__restrict__ E2, const double *__restrict__ alpha,
@@ -365,7 +365,6 @@ __global__ void k_dp_init_residual(const double *__restrict__ E2, const double *
                 const double Amu = a > 0.0 ? mu2[i] * d - acc_value(v.acc[k], j, fixed) - (double)rec[j] : 0.0;
                 const double rr = a > 0.0 ? E2[i] - Amu : 0.0;
                 r2[i] = rr;
-                v.acc[k][j] = 0.0;
                 red[2 * k] += rr * a * rr;
                 red[2 * k + 1] += a * rr * a * rr;
             }
@@ -405,7 +404,7 @@ __global__ void k_dp_direction(const double *__restrict__ r2, const double *__re
     }
 }
 
-// q_k = A p_k; partial p_k.q_k; clears the accumulators. The last block sets gamma_k.
+// q_k = A p_k; partial p_k.q_k. The last block sets gamma_k.
 template <class T>
 __global__ void k_dp_apply(const typename V4<T>::type *__restrict__ p2, const double *__restrict__ dg, DpVecs v,
                            int n_pad, double *__restrict__ q2, double *__restrict__ part, DpState *st, int fixed) {
@@ -421,7 +420,6 @@ __global__ void k_dp_apply(const typename V4<T>::type *__restrict__ p2, const do
                 const size_t j = (size_t)c * n_pad + s;
                 const double qq = pp[c] * d - acc_value(v.acc[k], j, fixed) - (double)rec[j];
                 q2[(size_t)k * 3 * n_pad + j] = qq;
-                v.acc[k][j] = 0.0;
                 red[k] += pp[c] * qq;
             }
         }
@@ -513,8 +511,8 @@ __device__ __forceinline__ void dp_block_parts4(const F2 *a, double *part) {
         for (int k = 0; k < 4; ++k) part[k * gridDim.x + blockIdx.x] = t[k];
 }
 
-// r_k = E_k - A mu_k (formed in FP64 once per solve, stored in FP32); clears the accumulators
-// and the directions; partial r.z and z.z of both systems. The last block sets the state.
+// r_k = E_k - A mu_k (formed in FP64 once per solve, stored in FP32); clears the
+// directions; partial r.z and z.z of both systems. The last block sets the state.
 __global__ void k_dp_init_residual_f(const double *__restrict__ E2, const float2 *__restrict__ dga,
                                      const float4 *__restrict__ mu2, DpVecs v, int n_pad, int n,
                                      float4 *__restrict__ r2, float4 *__restrict__ p2, double *__restrict__ part,
@@ -532,7 +530,6 @@ __global__ void k_dp_init_residual_f(const double *__restrict__ E2, const float2
                 const size_t i = (size_t)k * 3 * n_pad + (size_t)c * n_pad + s, j = (size_t)c * n_pad + s;
                 const double Amu = d.y > 0.f ? (double)mv[c] * d.x - acc_value(v.acc[k], j, fixed) - (double)rec[j] : 0.0;
                 rv[c] = d.y > 0.f ? (float)(E2[i] - Amu) : 0.f;
-                v.acc[k][j] = 0.0;
                 const float z = d.y * rv[c];
                 f2_add_prod(red[2 * k], rv[c], z);
                 f2_add_prod(red[2 * k + 1], z, z);
@@ -565,7 +562,7 @@ __global__ void k_dp_direction_f(const float4 *__restrict__ r2, const float2 *__
     }
 }
 
-// q_k = A p_k; partial p_k.q_k; clears the accumulators. The last block sets gamma_k.
+// q_k = A p_k; partial p_k.q_k. The last block sets gamma_k.
 __global__ void k_dp_apply_f(const float4 *__restrict__ p2, const float2 *__restrict__ dga, DpVecs v, int n_pad,
                              float4 *__restrict__ q2, double *__restrict__ part, DpState *st, int fixed) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
@@ -580,7 +577,6 @@ __global__ void k_dp_apply_f(const float4 *__restrict__ p2, const float2 *__rest
             for (int c = 0; c < 3; ++c) {
                 const size_t j = (size_t)c * n_pad + s;
                 qq[c] = fmaf(pp[c], d, -acc_f32(v.acc[k], j, fixed)) - rec[j];
-                v.acc[k][j] = 0.0;
                 f2_add_prod(red[k], pp[c], qq[c]);
             }
             q2[(size_t)k * n_pad + s] = make_float4(qq[0], qq[1], qq[2], 0.f);
@@ -776,8 +772,6 @@ int solve_t(ap_ctx *ctx, const double *gd, const double *gp, double tol, int max
         return ap_fail(ctx, AP_ERR_ARG, "induced_dipoles_pcg_dp cannot be captured into a graph");
     const int nb = ap_grid_for(ctx->n_pad, NT);
     AP_CUDA(cudaMemsetAsync(B->st, 0, sizeof(DpState), s));
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, s));
-    AP_CUDA(cudaMemsetAsync(B->acc2, 0, sizeof(double) * 3 * ctx->n_pad, s));
     constexpr bool F32 = std::is_same<T, float>::value;   // FP32 vectors (mixed and fixed modes)
     if (F32)
         k_dp_guess_f<<<nb, NT, 0, s>>>(gd, gp, B->E2, ctx->alpha, ctx->perm, ctx->n, ctx->n_pad, B->mu2f,
@@ -1186,15 +1180,10 @@ int dp_forces(ap_ctx *ctx, const double *d_mu_d, const double *d_mu_p, double *d
     return AP_OK;
 }
 
-// the two-set real-space product on the current directions alone (timing), or (clear) a
-// reset of the second accumulator afterwards
-int dp_matvec2_launch(ap_ctx *ctx, cudaStream_t s, int clear) {
+// the two-set real-space product on the current directions alone (timing)
+int dp_matvec2_launch(ap_ctx *ctx, cudaStream_t s) {
     if (!ctx->dp) return ap_fail(ctx, AP_ERR_STATE, "set_scaled_pairs() must come first");
     DpBuffers *B = dpb(ctx);
-    if (clear) {
-        AP_CUDA(cudaMemsetAsync(B->acc2, 0, sizeof(double) * 3 * ctx->n_pad, s));
-        return AP_OK;
-    }
     const size_t t4 = (ctx->prec == AP_FP64 ? sizeof(double) : sizeof(float)) * 4;
     const char *p0 = (const char *)B->p2;
     return real_matvec2_launch(ctx, p0, p0 + t4 * ctx->n_pad, ctx->acc, B->acc2, s);

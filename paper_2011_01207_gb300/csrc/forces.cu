@@ -21,7 +21,9 @@
 // accumulated per block in FP64 (fixed point in AP_FIXED) into nine device slots.
 #include "common.cuh"
 #include "pair_math.cuh"
+#include "pair_walk.cuh"
 
+#include <algorithm>
 #include <cmath>
 #include <type_traits>
 
@@ -29,22 +31,6 @@ void unsort3(ap_ctx *ctx, const double *src, double *out, cudaStream_t s);
 
 namespace {
 
-// the twelve running sums of block I's atom s (force, dU/dd, dU/dQ) to the accumulators
-template <class PA>
-__device__ __forceinline__ void flush12(double *frc, double *gdip, double *gquad, int n_pad, int s,
-                                        const typename PA::run_t *a) {
-    for (int c = 0; c < 3; ++c) PA::run_flush(frc + c * n_pad + s, a[c]);
-    for (int c = 0; c < 3; ++c) PA::run_flush(gdip + c * n_pad + s, a[3 + c]);
-    for (int c = 0; c < 6; ++c) PA::run_flush(gquad + c * n_pad + s, a[6 + c]);
-}
-// one item's twelve sums of a chunk atom s (already scaled)
-template <class PA>
-__device__ __forceinline__ void flush12_item(double *frc, double *gdip, double *gquad, int n_pad, int s,
-                                             const typename PA::shared_t *a) {
-    for (int c = 0; c < 3; ++c) PA::item_flush(frc + c * n_pad + s, a[c]);
-    for (int c = 0; c < 3; ++c) PA::item_flush(gdip + c * n_pad + s, a[3 + c]);
-    for (int c = 0; c < 6; ++c) PA::item_flush(gquad + c * n_pad + s, a[6 + c]);
-}
 // FP64 value v added to slot k of an array of FP64 numbers or (fixed) fixed-point integers,
 // by the only thread that updates that slot
 __device__ __forceinline__ void add_plain(double *arr, size_t k, double v, int fixed) {
@@ -79,388 +65,312 @@ __device__ __forceinline__ void block_add9(V *v, double *acc) {
     }
 }
 
-// out_a = sum_b mu_b dE_b/dR_a for the field E(R) of a multipole (q, d, Q) at the origin
-template <class T>
-__device__ __forceinline__ void mu_dot_field_grad(T q, const T *d, const T *Q /*xx xy xz yy yz zz*/, const T *mu,
-                                                  T dx, T dy, T dz, T R1, T R2, T R3, T R4, T *out) {
-    const T R[3] = {dx, dy, dz};
-    const T QR[3] = {Q[0] * dx + Q[1] * dy + Q[2] * dz, Q[1] * dx + Q[3] * dy + Q[4] * dz,
-                     Q[2] * dx + Q[4] * dy + Q[5] * dz};
-    const T Qm[3] = {Q[0] * mu[0] + Q[1] * mu[1] + Q[2] * mu[2], Q[1] * mu[0] + Q[3] * mu[1] + Q[4] * mu[2],
-                     Q[2] * mu[0] + Q[4] * mu[1] + Q[5] * mu[2]};
-    const T muR = mu[0] * dx + mu[1] * dy + mu[2] * dz;
-    const T dR = d[0] * dx + d[1] * dy + d[2] * dz;
-    const T dmu = d[0] * mu[0] + d[1] * mu[1] + d[2] * mu[2];
-    const T RQR = QR[0] * dx + QR[1] * dy + QR[2] * dz;
-    const T muQR = mu[0] * QR[0] + mu[1] * QR[1] + mu[2] * QR[2];
-    const T cR = -q * muR * R2 + dmu * R2 - dR * muR * R3 + T(2.0 / 3.0) * muQR * R3 - RQR * muR * R4 * T(1.0 / 3.0);
-    const T cmu = q * R1 + dR * R2 + RQR * R3 * T(1.0 / 3.0);
-    const T cd = muR * R2;
-    const T cQm = -T(2.0 / 3.0) * R2;
-    const T cQR = T(2.0 / 3.0) * muR * R3;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) out[a] = cR * R[a] + cmu * mu[a] + cd * d[a] + cQm * Qm[a] + cQR * QR[a];
-}
-
-// One warp per work item, pair sides walked in place as in the real-space field kernels: every
-// in-range pair gives the side (target t, source s) for both atoms, and with
-// R = x_t - x_s the same expressions give t's force and t's dU/dd, dU/dQ. Per side the
-// kernel accumulates, without the constant factors,
-//   F_t / f         += mu_t.G(R; M_s) - mu_s.G(R; q_t, -d_t, Q_t) + d(mu_t T mu_s)/dR
-//   dU/dd_t / (-f)  += -R_1 mu_s + R_2 (mu_s.R) R
-//   dU/dQ_t / (-f/3) += R_2 sym(mu_s R) - R_3 (mu_s.R) R R
-// so the pair's force is evaluated once per side (twice per pair) in exchange for lanes
-// that only ever see in-range pairs. In FP32 a lane takes two sides per step with their
-// radial terms in packed f32x2 arithmetic (fo_walk_x2): 255.9 -> 229.9 us at 96,000 atoms,
-// at 96 registers and 5 CTAs per SM (the same walk at 80 registers, 6 per SM, spilled more
-// and took 243.7 us).
-template <class T, class A>
-struct FoSmem {
-    typename V4<T>::type pos[64];   // x, y, z, Thole factor: [0,32) block I, [32,64) the item's j atoms
-    typename V4<T>::type qd[64];    // charge, dipole
-    typename V4<T>::type qa[64];    // Qxx, Qxy, Qxz, Qyy
-    typename V4<T>::type mu[64];    // induced dipole
-    T qb[2][64];                    // Qyz, Qzz
-    A acc[12][64];                  // per-target sums of the item
-    unsigned ex[32];                // exclusion words: lane i, bit j
-    unsigned words[64];             // pair bits: rows of the i atoms, then columns of the j atoms
+// ---- real space ----------------------------------------------------------------------------
+// One CTA per block of 32 atoms over the pair lists (pair_walk.cuh). What a target's force and
+// torque need of its neighbours are derivatives of two fields at the target: E of the induced
+// dipoles, up to second order, for the target's charge, dipole and quadrupole, and G, the first
+// derivative of the field of permanent multipoles and induced dipoles together, for its induced
+// dipole. So the walk accumulates those 30 numbers per target (as the smooth-PME part does) and
+// the target's own multipoles enter once at the end, instead of contracting two multipoles per
+// pair side: fewer operations, and no target multipoles in the walk's registers.
+// With R = x_target - x_source, u = mu.R, D = d + mu:
+//   E_a = -R1 mu_a + R2 u R_a
+//   E_ab = y_a R_b + y_b R_a + delta_ab sum R2 u,            y = R2 mu - (1/2) R3 u R
+//   E_abc = sym(w_a R_b R_c) + (V_a delta_bc + V_b delta_ac + V_c delta_ab),
+//           w = (1/3) R4 u R - R3 mu,                        V = R2 mu - R3 u R
+//   G_ab = t_a R_b + t_b R_a - (2/3) R2 Q_ab + delta_ab (q R1 + R2 D.R + (1/3) R3 R.Q.R),
+//           t = R2 D + (2/3) R3 Q R - (1/2) (q R2 + R3 D.R + (1/3) R4 R.Q.R) R
+// and then
+//   F_c / f = q E_c + sum_a d_a E_ac + (1/3) sum_ab Q_ab E_abc + sum_a mu_a G_ac
+//   dU/dd / (-f) = E,   dU/dQ / (-f/3) = E_ab without its trace part (Q is traceless).
+// Measured on GB300 (ncu, warm): 228 -> 134.7 us at 96,000 atoms, 44.2 -> 23.5 us at 6,000, against
+// contracting both atoms' multipoles per pair side on 32 x 32 pair masks. 159 registers, so 3 CTAs
+// per SM (shared memory would hold 4): what bounds it is issue at that occupancy.
+// Every term is linear in the R_n, which come negated, so the sums are those of -E and -G.
+// Excluded pairs (sigma = 0 between permanent and induced, 1 between induced and induced) come
+// first in the lists and take two sets of radial functions.
+template <class V>
+struct FieldSums {
+    V E[3], xx, yy, zz, xy, xz, yz, tr;              // the diagonal of E_ab halved
+    V S[10], W[3];                                   // xxx yyy zzz (a third) xxy xxz xyy yyz xzz yzz xyz; V
+    V gxx, gyy, gzz, gxy, gxz, gyz, gtr;             // G: the diagonal's t_a R_a part halved
+    V qxx, qyy, qzz;                                 // and the diagonal of -(2/3) R2 Q
 };
+constexpr int FS = 33;
 
 template <class T>
-constexpr int fo_warps() { return sizeof(T) == 4 ? 4 : 2; }
+__device__ __forceinline__ void zero_sums(FieldSums<typename Vec<T>::type> &a) {
+    typename Vec<T>::type *v = reinterpret_cast<typename Vec<T>::type *>(&a);
+#pragma unroll
+    for (int k = 0; k < FS; ++k) v[k] = splat2(T(0));
+}
 
-// the target atom of a pair side: position and Thole factor, charge and dipole, quadrupole
+// the induced dipole mu's share of E, E_ab and E_abc (radial functions Rn[0..3])
 template <class T>
-struct FoTarget {
-    typename V4<T>::type pos, qd, qa, mu;
-    T qyz, qzz;
+__device__ __forceinline__ void add_induced(FieldSums<typename Vec<T>::type> &a, const typename Vec<T>::type *R,
+                                            const typename Vec<T>::type *Rn, const typename V4<T>::type &mu) {
+    typedef typename Vec<T>::type Vt;
+    const Vt mx = splat2(mu.x), my = splat2(mu.y), mz = splat2(mu.z);
+    const Vt u = fma2(mx, R[0], fma2(my, R[1], mul2(mz, R[2])));
+    const Vt u2 = mul2(Rn[1], u), u3 = mul2(Rn[2], u), n1 = mul2(Rn[0], splat2(T(-1)));
+    const Vt h3 = mul2(u3, splat2(T(-0.5))), n3 = mul2(u3, splat2(T(-1))), m3 = mul2(Rn[2], splat2(T(-1)));
+    const Vt u4 = mul2(mul2(Rn[3], u), splat2(T(1.0 / 3.0)));
+    a.E[0] = fma2(n1, mx, fma2(u2, R[0], a.E[0]));
+    a.E[1] = fma2(n1, my, fma2(u2, R[1], a.E[1]));
+    a.E[2] = fma2(n1, mz, fma2(u2, R[2], a.E[2]));
+    a.tr = add2(a.tr, u2);
+    const Vt sx = mul2(Rn[1], mx), sy = mul2(Rn[1], my), sz = mul2(Rn[1], mz);
+    const Vt yx = fma2(h3, R[0], sx), yy = fma2(h3, R[1], sy), yz = fma2(h3, R[2], sz);
+    a.xx = fma2(yx, R[0], a.xx);
+    a.yy = fma2(yy, R[1], a.yy);
+    a.zz = fma2(yz, R[2], a.zz);
+    a.xy = fma2(yx, R[1], fma2(yy, R[0], a.xy));
+    a.xz = fma2(yx, R[2], fma2(yz, R[0], a.xz));
+    a.yz = fma2(yy, R[2], fma2(yz, R[1], a.yz));
+    a.W[0] = add2(a.W[0], fma2(n3, R[0], sx));
+    a.W[1] = add2(a.W[1], fma2(n3, R[1], sy));
+    a.W[2] = add2(a.W[2], fma2(n3, R[2], sz));
+    const Vt wx = fma2(u4, R[0], mul2(m3, mx)), wy = fma2(u4, R[1], mul2(m3, my)), wz = fma2(u4, R[2], mul2(m3, mz));
+    const Vt rxx = mul2(R[0], R[0]), ryy = mul2(R[1], R[1]), rzz = mul2(R[2], R[2]);
+    const Vt rxy = mul2(R[0], R[1]), rxz = mul2(R[0], R[2]), ryz = mul2(R[1], R[2]);
+    const Vt wx2 = add2(wx, wx), wy2 = add2(wy, wy), wz2 = add2(wz, wz);
+    a.S[0] = fma2(wx, rxx, a.S[0]);
+    a.S[1] = fma2(wy, ryy, a.S[1]);
+    a.S[2] = fma2(wz, rzz, a.S[2]);
+    a.S[3] = fma2(wy, rxx, fma2(wx2, rxy, a.S[3]));   // xxy
+    a.S[4] = fma2(wz, rxx, fma2(wx2, rxz, a.S[4]));   // xxz
+    a.S[5] = fma2(wx, ryy, fma2(wy2, rxy, a.S[5]));   // xyy
+    a.S[6] = fma2(wz, ryy, fma2(wy2, ryz, a.S[6]));   // yyz
+    a.S[7] = fma2(wx, rzz, fma2(wz2, rxz, a.S[7]));   // xzz
+    a.S[8] = fma2(wy, rzz, fma2(wz2, ryz, a.S[8]));   // yzz
+    a.S[9] = fma2(wx, ryz, fma2(wy, rxz, fma2(wz, rxy, a.S[9])));   // xyz
+}
+
+// the share in G of a multipole (q, D, Q); POLES: with charge and quadrupole
+template <class T, bool POLES>
+__device__ __forceinline__ void add_gradient(FieldSums<typename Vec<T>::type> &a, const typename Vec<T>::type *R,
+                                             const typename Vec<T>::type *Rn, T q, T Dx, T Dy, T Dz,
+                                             const typename V4<T>::type &qa, T qyz, T qzz) {
+    typedef typename Vec<T>::type Vt;
+    const Vt dx = splat2(Dx), dy = splat2(Dy), dz = splat2(Dz);
+    const Vt DR = fma2(dx, R[0], fma2(dy, R[1], mul2(dz, R[2])));
+    Vt c = mul2(Rn[2], DR), tr = mul2(Rn[1], DR);
+    Vt tx = mul2(Rn[1], dx), ty = mul2(Rn[1], dy), tz = mul2(Rn[1], dz);
+    if (POLES) {
+        const Vt Qx = fma2(splat2(qa.x), R[0], fma2(splat2(qa.y), R[1], mul2(splat2(qa.z), R[2])));
+        const Vt Qy = fma2(splat2(qa.y), R[0], fma2(splat2(qa.w), R[1], mul2(splat2(qyz), R[2])));
+        const Vt Qz = fma2(splat2(qa.z), R[0], fma2(splat2(qyz), R[1], mul2(splat2(qzz), R[2])));
+        const Vt RQR = mul2(fma2(Qx, R[0], fma2(Qy, R[1], mul2(Qz, R[2]))), splat2(T(1.0 / 3.0)));
+        c = fma2(splat2(q), Rn[1], fma2(RQR, Rn[3], c));
+        tr = fma2(splat2(q), Rn[0], fma2(RQR, Rn[2], tr));
+        const Vt r3 = mul2(Rn[2], splat2(T(2.0 / 3.0))), r2 = mul2(Rn[1], splat2(T(-2.0 / 3.0)));
+        tx = fma2(r3, Qx, tx);
+        ty = fma2(r3, Qy, ty);
+        tz = fma2(r3, Qz, tz);
+        a.qxx = fma2(r2, splat2(qa.x), a.qxx);
+        a.qyy = fma2(r2, splat2(qa.w), a.qyy);
+        a.qzz = fma2(r2, splat2(qzz), a.qzz);
+        a.gxy = fma2(r2, splat2(qa.y), a.gxy);
+        a.gxz = fma2(r2, splat2(qa.z), a.gxz);
+        a.gyz = fma2(r2, splat2(qyz), a.gyz);
+    }
+    c = mul2(c, splat2(T(-0.5)));
+    tx = fma2(c, R[0], tx);
+    ty = fma2(c, R[1], ty);
+    tz = fma2(c, R[2], tz);
+    a.gtr = add2(a.gtr, tr);
+    a.gxx = fma2(tx, R[0], a.gxx);
+    a.gyy = fma2(ty, R[1], a.gyy);
+    a.gzz = fma2(tz, R[2], a.gzz);
+    a.gxy = fma2(tx, R[1], fma2(ty, R[0], a.gxy));
+    a.gxz = fma2(tx, R[2], fma2(tz, R[0], a.gxz));
+    a.gyz = fma2(ty, R[2], fma2(tz, R[1], a.gyz));
+}
+
+// a target's own multipoles: charge, dipole, quadrupole (xx xy xz yy yz zz) and induced dipole
+template <class X>
+struct OwnPoles {
+    X q, d[3], Q[6], mu[3];
 };
-template <class T, class SM>
-__device__ __forceinline__ void fo_target(const SM &S, int t, FoTarget<T> &g) {
-    g.pos = S.pos[t];
-    g.qd = S.qd[t];
-    g.qa = S.qa[t];
-    g.mu = S.mu[t];
-    g.qyz = S.qb[0][t];
-    g.qzz = S.qb[1][t];
+// force (over f) of those multipoles in the fields of the sums a[0..FS-1] (order of FieldSums)
+template <class X>
+__device__ __forceinline__ void own_force(const X *a, const OwnPoles<X> &m, X *F) {
+    const X tr = a[9], g = a[29];
+    const X Eab[3][3] = {{2 * a[3] + tr, a[6], a[7]}, {a[6], 2 * a[4] + tr, a[8]}, {a[7], a[8], 2 * a[5] + tr}};
+    const X G[3][3] = {{2 * a[23] + a[30] + g, a[26], a[27]}, {a[26], 2 * a[24] + a[31] + g, a[28]},
+                       {a[27], a[28], 2 * a[25] + a[32] + g}};
+    const X *S = a + 10, *W = a + 20, *Q = m.Q;
+    // sum_bc Q_bc E_abc, with sum_bc Q_bc delta_bc = 0
+    const X QS[3] = {Q[0] * 3 * S[0] + Q[3] * S[5] + Q[5] * S[7] + 2 * (Q[1] * S[3] + Q[2] * S[4] + Q[4] * S[9]),
+                     Q[0] * S[3] + Q[3] * 3 * S[1] + Q[5] * S[8] + 2 * (Q[1] * S[5] + Q[2] * S[9] + Q[4] * S[6]),
+                     Q[0] * S[4] + Q[3] * S[6] + Q[5] * 3 * S[2] + 2 * (Q[1] * S[9] + Q[2] * S[7] + Q[4] * S[8])};
+    const X QW[3] = {Q[0] * W[0] + Q[1] * W[1] + Q[2] * W[2], Q[1] * W[0] + Q[3] * W[1] + Q[4] * W[2],
+                     Q[2] * W[0] + Q[4] * W[1] + Q[5] * W[2]};
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+        F[c] = m.q * a[c] + m.d[0] * Eab[0][c] + m.d[1] * Eab[1][c] + m.d[2] * Eab[2][c] +
+               (QS[c] + 2 * QW[c]) * X(1.0 / 3.0) + m.mu[0] * G[0][c] + m.mu[1] * G[1][c] + m.mu[2] * G[2][c];
 }
 
-// one side's terms, given its R = x_target - x_source and its radial functions Rd (with the
-// pair's scale), Ru (unscaled): the force, dU/dd and dU/dQ of the target (unscaled sums), and
-// with VS the side's F R^T
-template <class T, bool VS, class SM>
-__device__ __forceinline__ void fo_side_terms(const SM &S, const FoTarget<T> &g, int src, T dx, T dy, T dz,
-                                              const T *Rd, const T *Ru, T *f, T *vs) {
+template <class T>
+struct PoleArgs {
+    const typename V4<T>::type *posw, *dipd, *quad0, *quad1, *mu;
+};
+template <class T>
+__device__ __forceinline__ OwnPoles<T> own_poles(const PoleArgs<T> &a, int s, int n) {
+    OwnPoles<T> m;
+    typename V4<T>::type d, c, e, u;
+    d.x = d.y = d.z = T(0);
+    c = e = u = d;
+    c.w = e.w = T(0);
+    if (s < n) {
+        d = a.dipd[s];
+        c = a.quad0[s];
+        e = a.quad1[s];
+        u = a.mu[s];
+    }
+    m.q = e.w;
+    m.d[0] = d.x; m.d[1] = d.y; m.d[2] = d.z;
+    m.Q[0] = c.x; m.Q[1] = c.y; m.Q[2] = c.z; m.Q[3] = c.w; m.Q[4] = e.x; m.Q[5] = e.y;
+    m.mu[0] = u.x; m.mu[1] = u.y; m.mu[2] = u.z;
+    return m;
+}
+
+constexpr int FT = 128;   // threads of a CTA
+
+// VIR: also the pairs' virial, sum over pairs of (dU/dR) R^T = -(1/2) sum over sides of F R^T,
+// which needs every side's own force: its share of the sums by itself, and the targets'
+// multipoles in registers.
+template <class T, int PARTS, bool VIR>
+__global__ void __launch_bounds__(FT, sizeof(T) == 4 && !VIR ? 3 : 1) k_pair_forces(
+    ListArgs la, PoleArgs<T> src, double *__restrict__ frc, double *__restrict__ gdip, double *__restrict__ gquad,
+    int n_pad, PairConsts<T> pc, double fconst, double *__restrict__ vir, int fixed) {
     typedef typename V4<T>::type T4;
-    const T4 om = S.qd[src], oa = S.qa[src], ou = S.mu[src];
-    const T oyz = S.qb[0][src], ozz = S.qb[1][src];
-    const T mt[3] = {g.mu.x, g.mu.y, g.mu.z}, ms[3] = {ou.x, ou.y, ou.z};
-    const T ds[3] = {om.y, om.z, om.w}, ndt[3] = {-g.qd.y, -g.qd.z, -g.qd.w};
-    const T Qs[6] = {oa.x, oa.y, oa.z, oa.w, oyz, ozz};
-    const T Qt[6] = {g.qa.x, g.qa.y, g.qa.z, g.qa.w, g.qyz, g.qzz};
-    T A[3], Bv[3];
-    mu_dot_field_grad<T>(om.x, ds, Qs, mt, dx, dy, dz, Rd[0], Rd[1], Rd[2], Rd[3], A);
-    mu_dot_field_grad<T>(g.qd.x, ndt, Qt, ms, dx, dy, dz, Rd[0], Rd[1], Rd[2], Rd[3], Bv);
-    const T mts = mt[0] * ms[0] + mt[1] * ms[1] + mt[2] * ms[2];
-    const T mtr = mt[0] * dx + mt[1] * dy + mt[2] * dz;
-    const T msr = ms[0] * dx + ms[1] * dy + ms[2] * dz;
-    const T cR = Ru[1] * mts - Ru[2] * mtr * msr;
-    const T R[3] = {dx, dy, dz};
-    T fs[3];
+    typedef typename Vec<T>::type Vt;
+    constexpr int W = Vec<T>::W;
+    extern __shared__ __align__(16) unsigned char raw[];
+    constexpr int ROW = (AP_CHUNK + 1) * (int)sizeof(T4);
+    typedef Layout<T, PARTS> LY;
+    const LY ly;
+    const RadialConsts<T> rk(pc);
+    Targets<T> tg;
+    tg.load(src.posw, ly.slot(), ly.h, pc.n, pc.rc2, rk.ta);
+    FieldSums<Vt> sum;
+    zero_sums<T>(sum);
+    OwnPoles<T> own[W];
+    Vt vs[9];                       // sum of F R^T over this thread's sides (VIR)
+    if constexpr (VIR) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        fs[k] = A[k] - Bv[k] + cR * R[k] + Ru[1] * (mt[k] * msr + ms[k] * mtr);
-        f[k] += fs[k];
-        f[3 + k] += -Rd[0] * ms[k] + Rd[1] * msr * R[k];
+        for (int h = 0; h < W; ++h) own[h] = own_poles<T>(src, ly.slot() + h, pc.n);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) vs[k] = splat2(T(0));
     }
-    if constexpr (VS) {
+    const T4 *const from[4] = {src.dipd, src.quad0, src.quad1, src.mu};
+    for_chunks<T, PARTS>(raw, la, ly, from, [&](const unsigned *list, int words, int flagged, int) {
+        auto side = [&](unsigned e, auto ex) {
+            constexpr bool EX = decltype(ex)::value;
+            const unsigned char *at = raw + (e & 0xfff0u) * (unsigned)(sizeof(T4) / 16);
+            const T4 o = *reinterpret_cast<const T4 *>(at), d = *reinterpret_cast<const T4 *>(at + ROW);
+            const T4 qa = *reinterpret_cast<const T4 *>(at + 2 * ROW), qb = *reinterpret_cast<const T4 *>(at + 3 * ROW);
+            const T4 mu = *reinterpret_cast<const T4 *>(at + 4 * ROW);
+            Vt R[3], Mu[4], Md[4], pen;
+            bool exa, exb;
+            const Vt r2 = tg.template vector<EX>(o, e, R, pen, exa, exb);
+            radial<4, EX>(rk, r2, mul1(tg.w, o.w), pen, exa, exb, Mu, Md);
+            auto add = [&](FieldSums<Vt> &a) {
+                add_induced<T>(a, R, EX ? Md : Mu, mu);
+                if constexpr (EX) {
+                    add_gradient<T, true>(a, R, Md, qb.w, d.x, d.y, d.z, qa, qb.x, qb.y);
+                    add_gradient<T, false>(a, R, Mu, T(0), mu.x, mu.y, mu.z, qa, T(0), T(0));
+                } else {
+                    add_gradient<T, true>(a, R, Mu, qb.w, d.x + mu.x, d.y + mu.y, d.z + mu.z, qa, qb.x, qb.y);
+                }
+            };
+            // in FP32 the sums take the same operations with and without the virial (in AP_FIXED the
+            // forces are the same bit for bit)
+            if constexpr (!VIR || W == 2) add(sum);
+            if constexpr (VIR) {
+                FieldSums<Vt> one;
+                zero_sums<T>(one);
+                add(one);
+                const Vt *o1 = reinterpret_cast<const Vt *>(&one);
+                if constexpr (W == 1) {
+                    Vt *t = reinterpret_cast<Vt *>(&sum);
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+                    for (int k = 0; k < FS; ++k) t[k] = add2(t[k], o1[k]);
+                }
 #pragma unroll
-            for (int b = 0; b < 3; ++b) vs[3 * a + b] += fs[a] * R[b];
-    }
-    const int ia[6] = {0, 0, 0, 1, 1, 2}, ib[6] = {0, 1, 2, 1, 2, 2};
+                for (int h = 0; h < W; ++h) {
+                    T v[FS], F[3];
 #pragma unroll
-    for (int k = 0; k < 6; ++k)
-        f[6 + k] += Rd[1] * (ms[ia[k]] * R[ib[k]] + R[ia[k]] * ms[ib[k]]) - Rd[2] * msr * R[ia[k]] * R[ib[k]];
-}
-
-// one side in full (scalar radial terms)
-template <class T, bool MINIMG, bool VS, class SM>
-__device__ __forceinline__ void fo_side(const SM &S, const PairConsts<T> &pc, const FoTarget<T> &g, int tg, int src,
-                                        T *f, T *vs) {
-    typedef typename V4<T>::type T4;
-    const int sl = src & 31;   // the source's lane within its half
-    const bool exb = tg < 32 ? (S.ex[tg] >> sl) & 1u : (S.ex[sl] >> (tg - 32)) & 1u;
-    const T4 o = S.pos[src];
-    T dx, dy, dz;
-    pair_vector<T, MINIMG>(pc, g.pos.x, g.pos.y, g.pos.z, o.x, o.y, o.z, T(0), T(0), T(0), dx, dy, dz);
-    const T r2 = dx * dx + dy * dy + dz * dz;
-    const T rinv = ap_rsqrt(r2), r = r2 * rinv, rinv2 = rinv * rinv;
-    T B[4], U[4], oml[4];
-    screened<T, 4>(pc, r, rinv, rinv2, B, U);
-    thole_oml<T, 4>(pc.thole_a * r2 * r * g.pos.w * o.w, oml);
-    T Rd[4], Ru[3];
+                    for (int k = 0; k < FS; ++k) v[k] = Vec<T>::get(o1[k], h);
+                    own_force<T>(v, own[h], F);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) Rd[k] = B[k] - (exb ? U[k] : oml[k] * U[k]);
+                    for (int x = 0; x < 3; ++x)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) Ru[k] = B[k] - oml[k] * U[k];
-    fo_side_terms<T, VS>(S, g, src, dx, dy, dz, Rd, Ru, f, vs);
-}
-
-// The walk over a lane's share of the item's sides (plain stores on leaving a target, the last
-// target left in `cur` for the caller's atomic add)
-template <class T, bool MINIMG, bool VS, class PA, class SM>
-__device__ __forceinline__ void fo_walk(SM &S, SideSlice &slice, const PairConsts<T> &pc, const T *scf, int &cur,
-                                        T *f, T *vs) {
-    FoTarget<T> g;
-    while (slice.left > 0) {
-        int tg, src;
-        slice.next(S.words, tg, src);
-        if (tg != cur) {
-            if (cur >= 0) {   // the only lane that leaves this target: a plain store
-#pragma unroll
-                for (int k = 0; k < 12; ++k) PA::shared_put(&S.acc[k][cur], f[k] * scf[k]);
-            }
-#pragma unroll
-            for (int k = 0; k < 12; ++k) f[k] = T(0);
-            cur = tg;
-            fo_target<T>(S, tg, g);
-        }
-        fo_side<T, MINIMG, VS>(S, pc, g, tg, src, f, vs);
-    }
-}
-
-// FP32: two consecutive sides per step, their radial terms in packed f32x2 arithmetic
-// (radial_forces_x2), the multipole terms per side; an odd last side takes the scalar path
-template <bool MINIMG, bool VS, class PA, class SM>
-__device__ __forceinline__ void fo_walk_x2(SM &S, SideSlice &slice, const PairConsts<float> &pc,
-                                           const PairConsts2 &k, const float *scf, int &cur, float *f, float *vs) {
-    FoTarget<float> g;
-    auto enter = [&](int t) {
-        if (cur >= 0) {   // the only lane that leaves this target: a plain store
-#pragma unroll
-            for (int q = 0; q < 12; ++q) PA::shared_put(&S.acc[q][cur], f[q] * scf[q]);
-        }
-#pragma unroll
-        for (int q = 0; q < 12; ++q) f[q] = 0.f;
-        cur = t;
-        fo_target<float>(S, t, g);
-    };
-    while (slice.left > 1) {
-        int ta, sa, tb, sb;
-        slice.next(S.words, ta, sa);
-        slice.next(S.words, tb, sb);
-        if (ta != cur) enter(ta);
-        const float4 pb = tb == ta ? g.pos : S.pos[tb];
-        const int la = sa & 31, lb = sb & 31;
-        const bool exa = ta < 32 ? (S.ex[ta] >> la) & 1u : (S.ex[la] >> (ta - 32)) & 1u;
-        const bool exb = tb < 32 ? (S.ex[tb] >> lb) & 1u : (S.ex[lb] >> (tb - 32)) & 1u;
-        const float4 oa = S.pos[sa], ob = S.pos[sb];
-        float dxa, dya, dza, dxb, dyb, dzb;
-        pair_vector<float, MINIMG>(pc, g.pos.x, g.pos.y, g.pos.z, oa.x, oa.y, oa.z, 0.f, 0.f, 0.f, dxa, dya, dza);
-        pair_vector<float, MINIMG>(pc, pb.x, pb.y, pb.z, ob.x, ob.y, ob.z, 0.f, 0.f, 0.f, dxb, dyb, dzb);
-        const float2 dx = make_float2(dxa, dxb), dy = make_float2(dya, dyb), dz = make_float2(dza, dzb);
-        const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
-        float2 Rd2[4], Ru2[3];
-        radial_forces_x2(k, r2, make_float2(g.pos.w * oa.w, pb.w * ob.w), exa, exb, Rd2, Ru2);
-        {
-            const float Rd[4] = {Rd2[0].x, Rd2[1].x, Rd2[2].x, Rd2[3].x}, Ru[3] = {Ru2[0].x, Ru2[1].x, Ru2[2].x};
-            fo_side_terms<float, VS>(S, g, sa, dxa, dya, dza, Rd, Ru, f, vs);
-        }
-        if (tb != cur) enter(tb);
-        {
-            const float Rd[4] = {Rd2[0].y, Rd2[1].y, Rd2[2].y, Rd2[3].y}, Ru[3] = {Ru2[0].y, Ru2[1].y, Ru2[2].y};
-            fo_side_terms<float, VS>(S, g, sb, dxb, dyb, dzb, Rd, Ru, f, vs);
-        }
-    }
-    if (slice.left > 0) {
-        int tg, src;
-        slice.next(S.words, tg, src);
-        if (tg != cur) enter(tg);
-        fo_side<float, MINIMG, VS>(S, pc, g, tg, src, f, vs);
-    }
-}
-
-// VIR: also the pairs' virial. Without per-pair minimum image every position of an item is
-// relative to block I's origin, and the item holds both sides of each of its pairs, whose
-// forces are opposite; so the item's sum over pairs of (dU/dR) R^T = -sum over sides of
-// F_t R^T / 2 equals -sum over its 64 targets of F_t x_t^T, formed once per item from the
-// per-target sums the kernel keeps anyway. With per-pair minimum image (small boxes) the
-// sides' F R^T are summed as they come.
-template <class T, bool MINIMG, bool FX, bool VIR>
-__global__ void __launch_bounds__(128, VIR ? 4 : 5) k_pair_forces(
-    WorkArgs wa, const typename V4<T>::type *__restrict__ posq,
-    const typename V4<T>::type *__restrict__ dipd, const typename V4<T>::type *__restrict__ quad0,
-    const typename V4<T>::type *__restrict__ quad1, const typename V4<T>::type *__restrict__ muv,
-    double *__restrict__ frc, double *__restrict__ gdip, double *__restrict__ gquad, int n_pad, PairConsts<T> pc,
-    double fconst, double *__restrict__ vir) {
-    typedef typename V4<T>::type T4;
-    typedef PairAcc<T, FX> PA;
-    __shared__ FoSmem<T, typename PA::shared_t> smem[fo_warps<T>()];
-    FoSmem<T, typename PA::shared_t> &S = smem[threadIdx.x >> 5];
-    const int lane = threadIdx.x & 31;
-    PairConsts2 k2;
-    if constexpr (std::is_same<T, float>::value) k2 = make_consts2(pc);
-    const long gw = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long nw = ((long)gridDim.x * blockDim.x) >> 5;
-    long t0, t1;
-    work_range(wa, gw, nw, t0, t1);
-    const T4 *cpos = (const T4 *)wa.chunk_pos;
-    const double sc[12] = {fconst, fconst, fconst, -fconst, -fconst, -fconst, -fconst / 3, -fconst / 3,
-                           -fconst / 3, -fconst / 3, -fconst / 3, -fconst / 3};
-    // FP64 mode: per-item sums are unscaled and scaled in FP64; mixed and fixed point: scaled
-    // in T as they enter the item's sums (so that no FP64 multiply runs per item, and the
-    // fixed-point integers hold the final quantities)
-    constexpr bool PRESCALE = FX || sizeof(T) == 4;
-    T scf[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) scf[k] = PRESCALE ? (T)sc[k] : T(1);
-    int curI = -1;
-    typename PA::run_t ai[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) PA::run_zero(ai[k]);
-    typedef typename std::conditional<FX, long long, double>::type vacc_t;
-    vacc_t vacc[9];                 // this lane's share of the virial (VIR)
-#pragma unroll
-    for (int k = 0; k < 9; ++k) vacc[k] = 0;
-    for (long t = t0; t < t1; ++t) {
-        const int2 it = wa.work[t];
-        __syncwarp();
-        if (it.x != curI) {
-            if (curI >= 0 && curI * 32 + lane < pc.n) flush12<PA>(frc, gdip, gquad, n_pad, curI * 32 + lane, ai);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) PA::run_zero(ai[k]);
-            curI = it.x;
-            const int si = curI * 32 + lane;
-            const T4 a = posq[si], b = dipd[si], c = quad0[si], d = quad1[si];
-            T4 p, m;
-            p.x = a.x; p.y = a.y; p.z = a.z; p.w = b.w;
-            m.x = a.w; m.y = b.x; m.z = b.y; m.w = b.z;
-            S.pos[lane] = p;
-            S.qd[lane] = m;
-            S.qa[lane] = c;
-            S.mu[lane] = muv[si];
-            S.qb[0][lane] = d.x;
-            S.qb[1][lane] = d.y;
-        }
-        const bool diag = it.y < 0;
-        int sj = -1;
-        unsigned ex;
-        if (diag) {
-            S.pos[32 + lane] = S.pos[lane];
-            S.qd[32 + lane] = S.qd[lane];
-            S.qa[32 + lane] = S.qa[lane];
-            S.mu[32 + lane] = S.mu[lane];
-            S.qb[0][32 + lane] = S.qb[0][lane];
-            S.qb[1][32 + lane] = S.qb[1][lane];
-            const int e = wa.tile_excl[wa.tile_off[curI]];
-            ex = e >= 0 ? wa.excl_mask[(size_t)e * 32 + lane] : 0u;
-        } else {
-            const size_t cs = (size_t)it.y * 32 + lane;
-            sj = wa.chunk_j[cs];
-            S.pos[32 + lane] = cpos[cs];
-            T4 m, c, d, u;
-            m.x = m.y = m.z = m.w = T(0);
-            c = m;
-            d = m;
-            u = m;
-            if (sj >= 0) {
-                const T4 a = posq[sj], b = dipd[sj];
-                c = quad0[sj];
-                d = quad1[sj];
-                u = muv[sj];
-                m.x = a.w; m.y = b.x; m.z = b.y; m.w = b.z;
-            }
-            S.qd[32 + lane] = m;
-            S.qa[32 + lane] = c;
-            S.mu[32 + lane] = u;
-            S.qb[0][32 + lane] = d.x;
-            S.qb[1][32 + lane] = d.y;
-            ex = wa.chunk_flag[it.y] ? wa.chunk_mask[cs] : 0u;
-        }
-        S.ex[lane] = ex;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            S.acc[k][lane] = 0;
-            S.acc[k][32 + lane] = 0;
-        }
-        SideSlice slice;
-        slice.load(wa.pmask[(size_t)t * 32 + lane], wa.pmask_t[(size_t)t * 32 + lane], wa.pstart[(size_t)t * 32 + lane],
-                 lane, S.words);
-        int cur = -1;
-        T f[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) f[k] = T(0);
-        T vs[9];                    // sum of F_side R^T over this lane's sides (VIR, MINIMG)
-#pragma unroll
-        for (int k = 0; k < 9; ++k) vs[k] = T(0);
-        if constexpr (std::is_same<T, float>::value)
-            fo_walk_x2<MINIMG, VIR && MINIMG, PA>(S, slice, pc, k2, scf, cur, f, vs);
-        else
-            fo_walk<T, MINIMG, VIR && MINIMG, PA>(S, slice, pc, scf, cur, f, vs);
-        __syncwarp();   // the plain stores land before the last targets are added
-        if (cur >= 0) {
-#pragma unroll
-            for (int k = 0; k < 12; ++k) PA::shared_add(&S.acc[k][cur], f[k] * scf[k]);
-        }
-        __syncwarp();
-        if constexpr (VIR) {
-            // in kcal/mol: each side's force is f times the kernel's sums, the pair's virial half
-            // the sum over its two sides
-            double v[9];
-            if constexpr (MINIMG) {
-#pragma unroll
-                for (int k = 0; k < 9; ++k) v[k] = -0.5 * fconst * (double)vs[k];
-            } else {
-#pragma unroll
-                for (int k = 0; k < 9; ++k) v[k] = 0.0;
-                const bool oki = curI * 32 + lane < pc.n;          // padding slots hold NaN positions
-                const bool okj = diag ? oki : sj >= 0;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const int tt = h ? 32 + lane : lane;
-                    if (!(h ? okj : oki)) continue;
-                    const T4 ps = S.pos[tt];
-                    const double x[3] = {(double)ps.x, (double)ps.y, (double)ps.z};
-                    double F[3];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a)
-                        F[a] = FX ? ap_from_fx((long long)S.acc[a][tt])
-                                  : (PRESCALE ? 1.0 : sc[a]) * (double)S.acc[a][tt];
-#pragma unroll
-                    for (int a = 0; a < 3; ++a)
-#pragma unroll
-                        for (int b = 0; b < 3; ++b) v[3 * a + b] -= F[a] * x[b];
+                        for (int y = 0; y < 3; ++y) {
+                            T *t = reinterpret_cast<T *>(&vs[3 * x + y]) + h;
+                            *t = fma(F[x], Vec<T>::get(R[y], h), *t);
+                        }
                 }
             }
+        };
+        walk(list, words, flagged, ly.first, ly.STRIDE, [&](unsigned e) { side(e, std::true_type()); },
+             [&](unsigned e) { side(e, std::false_type()); });
+    });
+    // the sums of a target's threads through shared memory (the staged candidates are done with):
+    // number k of target h at red[(W k + h) FT + tid]
+    __syncthreads();
+    T *red = reinterpret_cast<T *>(raw), *tot = red + W * FS * FT;
+    {
+        const Vt *v = reinterpret_cast<const Vt *>(&sum);
 #pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                if constexpr (FX) vacc[k] += ap_to_fx(v[k]);
-                else vacc[k] += v[k];
-            }
+        for (int k = 0; k < FS; ++k)
+#pragma unroll
+            for (int h = 0; h < W; ++h) red[(W * k + h) * FT + threadIdx.x] = Vec<T>::get(v[k], h);
+    }
+    __syncthreads();
+    constexpr int NT = 2 * LY::PAIRS;   // targets of this CTA
+    for (int q = threadIdx.x; q < FS * NT; q += FT) {
+        const int k = q / NT, t = q % NT, pp = t >> 1, h = t & 1;
+        const T *r = red + (W == 2 ? 2 * k + h : k) * FT + pp * LY::TP + (W == 2 ? 0 : h);
+        T v = T(0);
+#pragma unroll
+        for (int i = 0; i < LY::TP; i += W == 2 ? 1 : 2) v += r[i];
+        tot[t * (FS + 1) + k] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < NT) {
+        const int t = threadIdx.x, slot = ly.I * 32 + (int)(blockIdx.x % PARTS) * NT + t;
+        T a[FS], F[3];
+#pragma unroll
+        for (int k = 0; k < FS; ++k) a[k] = tot[t * (FS + 1) + k];
+        own_force<T>(a, own_poles<T>(src, slot, pc.n), F);
+        const double f = fconst, g = fconst / 3;
+        for (int c = 0; c < 3; ++c) {
+            store_acc<double>(frc + (size_t)c * n_pad + slot, -f * (double)F[c], fixed);
+            store_acc<double>(gdip + (size_t)c * n_pad + slot, f * (double)a[c], fixed);
         }
-        typename PA::shared_t ti[12], tj[12];
+        const T Q[6] = {2 * a[3], a[6], a[7], 2 * a[4], a[8], 2 * a[5]};   // xx xy xz yy yz zz
+        for (int c = 0; c < 6; ++c) store_acc<double>(gquad + (size_t)c * n_pad + slot, g * (double)Q[c], fixed);
+    }
+    if constexpr (VIR) {
+        double v[9];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            ti[k] = S.acc[k][lane];
-            tj[k] = S.acc[k][32 + lane];
-            if constexpr (!PRESCALE) {
-                ti[k] *= sc[k];
-                tj[k] *= sc[k];
-            }
+        for (int k = 0; k < 9; ++k) {
+            double t = (double)Vec<T>::get(vs[k], 0);
+            if (W == 2) t += (double)Vec<T>::get(vs[k], 1);
+            v[k] = 0.5 * fconst * t;
         }
+        if (fixed) {
+            long long vf[9];
 #pragma unroll
-        for (int k = 0; k < 12; ++k) PA::run_add(ai[k], ti[k]);
-        if (diag) {
-#pragma unroll
-            for (int k = 0; k < 12; ++k) PA::run_add(ai[k], tj[k]);
-        } else if (sj >= 0) {
-            flush12_item<PA>(frc, gdip, gquad, n_pad, sj, tj);
+            for (int k = 0; k < 9; ++k) vf[k] = ap_to_fx(v[k]);
+            block_add9<FT>(vf, vir);
+        } else {
+            block_add9<FT>(v, vir);
         }
     }
-    if (curI >= 0 && curI * 32 + lane < pc.n) flush12<PA>(frc, gdip, gquad, n_pad, curI * 32 + lane, ai);
-    if constexpr (VIR) block_add9<32 * fo_warps<T>()>(vacc, vir);
 }
 
 // reciprocal-space gradient and source terms per atom
@@ -728,43 +638,29 @@ __global__ void k_unsort3_fx(const double *__restrict__ src, int n_pad, const in
     for (int c = 0; c < 3; ++c) out[3 * i + c] = acc_value(src, (size_t)c * n_pad + s, 1);
 }
 
-// the real-space force kernel over the current work items with the dipoles in ctx->p and
-// the multipoles (posq q, dipd, quad0, quad1) given, accumulating into frc, gdip and gquad;
-// with vir given, also the pairs' virial into vir[0..8]
-template <class T>
-int pair_forces_t(ap_ctx *ctx, cudaStream_t s, const void *posq, const void *dipd, const void *quad0,
-                  const void *quad1, double *frc, double *gdip, double *gquad, double *vir = nullptr) {
-    typedef typename V4<T>::type T4;
-    PairConsts<T> pc;
-    const ap_params &P = ctx->prm;
-    const double b = P.ewald_beta;
-    pc.beta = (T)b;
-    pc.c[0] = 0;
-    for (int k = 1; k <= 4; ++k) pc.c[k] = (T)(std::pow(2.0 * b * b, k) / (b * AP_SQRT_PI));
-    pc.thole_a = (T)P.thole_a;
-    pc.rc2 = (T)(P.cutoff * P.cutoff);
-    for (int dd = 0; dd < 3; ++dd) { pc.L[dd] = (T)P.box[dd]; pc.iL[dd] = (T)(1.0 / P.box[dd]); }
-    pc.n = ctx->n;
-    typedef void (*Kern)(WorkArgs, const T4 *, const T4 *, const T4 *, const T4 *, const T4 *, double *, double *,
-                         double *, int, PairConsts<T>, double, double *);
-    static const Kern kerns[8] = {k_pair_forces<T, false, false, false>, k_pair_forces<T, true, false, false>,
-                                  k_pair_forces<T, false, true, false>,  k_pair_forces<T, true, true, false>,
-                                  k_pair_forces<T, false, false, true>,  k_pair_forces<T, true, false, true>,
-                                  k_pair_forces<T, false, true, true>,   k_pair_forces<T, true, true, true>};
-    const int which = ctx->minimg + 2 * ctx->fixed + 4 * (vir ? 1 : 0);
-    const Kern kern = kerns[which];
-    static int grids[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    int &grid = grids[which];
-    if (!grid) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * fo_warps<T>(), 0);
-        grid = std::max(1, per_sm) * ctx->sm_count;
-    }
-    kern<<<grid, 32 * fo_warps<T>(), 0, s>>>(work_args(ctx), (const T4 *)posq, (const T4 *)dipd,
-                                            (const T4 *)quad0, (const T4 *)quad1, (const T4 *)ctx->p,
-                                            frc, gdip, gquad, ctx->n_pad, pc, AP_COULOMB, vir);
+// the real-space force kernel over the current pair lists with the dipoles in ctx->p and the
+// multipoles (dipd, quad0, quad1) given, written to frc, gdip and gquad; with vir given, also the
+// pairs' virial added to vir[0..8]
+template <class T, int PARTS>
+int pair_forces_p(ap_ctx *ctx, cudaStream_t s, const PoleArgs<T> &src, double *frc, double *gdip, double *gquad,
+                  double *vir) {
+    auto kern = vir ? k_pair_forces<T, PARTS, true> : k_pair_forces<T, PARTS, false>;
+    // the candidates' rows, or the reduction of the sums
+    const size_t bytes = std::max(5 * (AP_CHUNK + 1) * sizeof(typename V4<T>::type),
+                                  sizeof(T) * (Vec<T>::W * FS * FT + 32 * (FS + 1)));
+    AP_CUDA(allow_smem(kern, bytes));
+    kern<<<ctx->n_blocks * PARTS, FT, bytes, s>>>(list_args(ctx), src, frc, gdip, gquad, ctx->n_pad, make_consts<T>(ctx),
+                                                  AP_COULOMB, vir, ctx->fixed);
     AP_CUDA(cudaGetLastError());
     return AP_OK;
+}
+template <class T>
+int pair_forces_t(ap_ctx *ctx, cudaStream_t s, const void *dipd, const void *quad0, const void *quad1,
+                  double *frc, double *gdip, double *gquad, double *vir = nullptr) {
+    typedef typename V4<T>::type T4;
+    const PoleArgs<T> src = {(const T4 *)ctx->posw, (const T4 *)dipd, (const T4 *)quad0, (const T4 *)quad1, (const T4 *)ctx->p};
+    return quarter_blocks(ctx) ? pair_forces_p<T, 4>(ctx, s, src, frc, gdip, gquad, vir)
+                               : pair_forces_p<T, 1>(ctx, s, src, frc, gdip, gquad, vir);
 }
 
 // `extra`, if given, runs on the force stream after the pair and reciprocal terms and before
@@ -784,20 +680,22 @@ int forces_t(ap_ctx *ctx, const double *d_mu, double *d_energy, double *d_forces
     // reciprocal-space potential derivatives on the second stream, concurrent with the
     // energy and the real-space pair forces (they write only gbuf and the grid); joined
     // before the kernels that update the force arrays per atom
-    AP_CUDA(cudaEventRecord(ctx->ev_fork, s));
-    AP_CUDA(cudaStreamWaitEvent(ctx->s1, ctx->ev_fork, 0));
-    int rc = pme_forces_derivs(ctx, ctx->p, ctx->gbuf, ctx->s1, vir);
+    const cudaStream_t aux = aux_stream(ctx, s, ctx->s1);
+    if (aux != s) {
+        AP_CUDA(cudaEventRecord(ctx->ev_fork, s));
+        AP_CUDA(cudaStreamWaitEvent(aux, ctx->ev_fork, 0));
+    }
+    int rc = pme_forces_derivs(ctx, ctx->p, ctx->gbuf, aux, vir);
     if (rc) return rc;
-    AP_CUDA(cudaMemsetAsync(ctx->frc, 0, sizeof(double) * 3 * n_pad, s));
-    AP_CUDA(cudaMemsetAsync(ctx->gdip, 0, sizeof(double) * 3 * n_pad, s));
-    AP_CUDA(cudaMemsetAsync(ctx->gquad, 0, sizeof(double) * 6 * n_pad, s));
     AP_CUDA(cudaMemsetAsync(ctx->red + 8, 0, sizeof(double), s));
     // energy
     k_energy<<<ap_grid_for(n_pad, 256), 256, 0, s>>>(ctx->mu_s, ctx->E, n_pad, -0.5 * f, ctx->red + 8, ctx->fixed);
-    rc = pair_forces_t<T>(ctx, s, ctx->posq, ctx->dipd, ctx->quad0, ctx->quad1, ctx->frc, ctx->gdip, ctx->gquad, vir);
+    rc = pair_forces_t<T>(ctx, s, ctx->dipd, ctx->quad0, ctx->quad1, ctx->frc, ctx->gdip, ctx->gquad, vir);
     if (rc) return rc;
-    AP_CUDA(cudaEventRecord(ctx->ev_join, ctx->s1));
-    AP_CUDA(cudaStreamWaitEvent(s, ctx->ev_join, 0));
+    if (aux != s) {
+        AP_CUDA(cudaEventRecord(ctx->ev_join, aux));
+        AP_CUDA(cudaStreamWaitEvent(s, ctx->ev_join, 0));
+    }
     auto krec = vir ? k_recip_forces<T, true> : k_recip_forces<T, false>;
     krec<<<ap_grid_for(n, 128), 128, 0, s>>>(ctx->gbuf, ctx->mu_s, (const T4 *)ctx->posq, (const T4 *)ctx->dipd,
                                             (const T4 *)ctx->quad0, (const T4 *)ctx->quad1, n, n_pad, f, self_coef,
@@ -837,14 +735,11 @@ int mutual_forces_t(ap_ctx *ctx, const double *d_mu, void *const *mz, double *gd
     const double self_coef = 4.0 * std::pow(ctx->prm.ewald_beta, 3) / (3.0 * AP_SQRT_PI);
     if (vir) AP_CUDA(cudaMemsetAsync(vir, 0, sizeof(double) * 9, s));
     k_mu_load<T><<<ap_grid_for(n_pad, 256), 256, 0, s>>>(d_mu, ctx->perm, n, n_pad, ctx->mu_s, (T4 *)ctx->p);
-    AP_CUDA(cudaMemsetAsync(ctx->frc, 0, sizeof(double) * 3 * n_pad, s));
-    AP_CUDA(cudaMemsetAsync(gd, 0, sizeof(double) * 3 * n_pad, s));
-    AP_CUDA(cudaMemsetAsync(gq, 0, sizeof(double) * 6 * n_pad, s));
     AP_CUDA(cudaEventRecord(ctx->ev_fork, s));
     AP_CUDA(cudaStreamWaitEvent(ctx->s1, ctx->ev_fork, 0));
     int rc = pme_forces_derivs_mu(ctx, ctx->p, ctx->gbuf, ctx->s1, vir);
     if (rc) return rc;
-    rc = pair_forces_t<T>(ctx, s, mz[0], mz[1], mz[2], mz[3], ctx->frc, gd, gq, vir);
+    rc = pair_forces_t<T>(ctx, s, mz[1], mz[2], mz[3], ctx->frc, gd, gq, vir);
     if (rc) return rc;
     AP_CUDA(cudaEventRecord(ctx->ev_join, ctx->s1));
     AP_CUDA(cudaStreamWaitEvent(s, ctx->ev_join, 0));
@@ -876,9 +771,9 @@ __global__ void k_virial_out(const double *__restrict__ a, const double *__restr
 
 int pair_forces_launch(ap_ctx *ctx, cudaStream_t s) {
     return ctx->prec == AP_FP64
-               ? pair_forces_t<double>(ctx, s, ctx->posq, ctx->dipd, ctx->quad0, ctx->quad1, ctx->frc, ctx->gdip,
+               ? pair_forces_t<double>(ctx, s, ctx->dipd, ctx->quad0, ctx->quad1, ctx->frc, ctx->gdip,
                                        ctx->gquad)
-               : pair_forces_t<float>(ctx, s, ctx->posq, ctx->dipd, ctx->quad0, ctx->quad1, ctx->frc, ctx->gdip,
+               : pair_forces_t<float>(ctx, s, ctx->dipd, ctx->quad0, ctx->quad1, ctx->frc, ctx->gdip,
                                       ctx->gquad);
 }
 

@@ -17,6 +17,7 @@
 // Units: A, fs, amu, kcal/mol; 1 kcal/mol/A on 1 amu accelerates by 4.184e-4 A/fs^2.
 #include "common.cuh"
 #include "pair_math.cuh"
+#include "pair_walk.cuh"
 
 #include <cmath>
 
@@ -153,87 +154,90 @@ __device__ __forceinline__ void lj_fs(T r2, T eps, T sig, T rc, T &V, T &f_over_
     f_over_r = (T(24) * eps * (T(2) * s6 * s6 - s6) / r - Fc) / r;
 }
 
-// one warp per work item (grid-stride): lane i of block I takes the pairs (i, j) of its row
-// word (each in-range pair of the configuration appears in exactly one row word), minus its
-// exclusion bits; j's position, parameters and slot come from shared memory. Forces into acc
-// [3][n_pad] (slot order, FP64 atomics), energy into *energy.
-template <class T, bool MINIMG>
-__global__ void __launch_bounds__(128) k_lj_forces(WorkArgs wa, const typename V4<T>::type *__restrict__ posq,
+// one CTA per block over the pair lists (pair_walk.cuh); of a pair's two sides the one whose
+// source has the higher slot is taken. Forces into acc [3][n_pad] (slot order, FP64 atomics),
+// energy into *energy.
+template <class T>
+__global__ void __launch_bounds__(128) k_lj_forces(ListArgs la, const typename V4<T>::type *__restrict__ posw,
                                                    const int *__restrict__ perm, const double *__restrict__ lj,
-                                                   int n, int n_pad, T rc, T Lx, T Ly, T Lz,
-                                                   double *__restrict__ acc, double *__restrict__ energy) {
+                                                   int n, int n_pad, T rc, double *__restrict__ acc,
+                                                   double *__restrict__ energy) {
     typedef typename V4<T>::type T4;
-    __shared__ T4 sp[4][32];
-    __shared__ T se[4][32], ss[4][32];
-    __shared__ int sl[4][32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long gw = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long nw = ((long)gridDim.x * blockDim.x) >> 5;
-    const long nitems = *wa.n_work;
-    const T4 *cpos = (const T4 *)wa.chunk_pos;
-    double e_sum = 0.0;
-    for (long t = gw; t < nitems; t += nw) {
-        const int2 it = wa.work[t];
-        const int si = it.x * 32 + lane;
-        const bool vi = si < n;
-        const T4 pi = posq[si];
-        const T ei = vi ? (T)lj[2 * perm[si]] : T(0), sgi = vi ? (T)lj[2 * perm[si] + 1] : T(1);
-        int sj;
-        T4 pj;
-        unsigned ex;
-        if (it.y < 0) {
-            sj = si;
-            pj = pi;
-            const int e = wa.tile_excl[wa.tile_off[it.x]];
-            ex = e >= 0 ? wa.excl_mask[(size_t)e * 32 + lane] : 0u;
-        } else {
-            const size_t cs = (size_t)it.y * 32 + lane;
-            sj = wa.chunk_j[cs];
-            pj = cpos[cs];
-            ex = wa.chunk_flag[it.y] ? wa.chunk_mask[cs] : 0u;
-        }
-        const bool vj = sj >= 0 && sj < n;
-        __syncwarp();
-        sp[w][lane] = pj;
-        se[w][lane] = vj ? (T)lj[2 * perm[sj]] : T(0);
-        ss[w][lane] = vj ? (T)lj[2 * perm[sj] + 1] : T(1);
-        sl[w][lane] = vj ? sj : -1;
-        __syncwarp();
-        unsigned m = wa.pmask[(size_t)t * 32 + lane] & ~ex;
-        double fi[3] = {0.0, 0.0, 0.0};
-        while (m && vi && ei > T(0)) {
-            const int j = __ffs(m) - 1;
-            m &= m - 1u;
-            const T ej = se[w][j];
-            if (!(ej > T(0)) || sl[w][j] < 0) continue;
-            const T4 q = sp[w][j];
-            T dx = pi.x - q.x, dy = pi.y - q.y, dz = pi.z - q.z;
-            if (MINIMG) {
-                dx -= Lx * ap_rint(dx / Lx);
-                dy -= Ly * ap_rint(dy / Ly);
-                dz -= Lz * ap_rint(dz / Lz);
-            }
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            if (!(r2 < rc * rc)) continue;
-            // the pair function in FP64 (few pairs: oxygens only): the force-shifted terms of
-            // close and far pairs cancel in the sum, which FP32 would resolve to ~1e-5 only
-            const double ddx = dx, ddy = dy, ddz = dz;
-            double V, fr;
-            lj_fs<double>(ddx * ddx + ddy * ddy + ddz * ddz, sqrt((double)ei * (double)ej),
-                          0.5 * ((double)sgi + (double)ss[w][j]), (double)rc, V, fr);
-            e_sum += V;
-            const double f3[3] = {fr * ddx, fr * ddy, fr * ddz};
-            for (int c = 0; c < 3; ++c) {
-                fi[c] += f3[c];
-                atomicAdd(acc + (size_t)c * n_pad + sl[w][j], -f3[c]);
-            }
-        }
-        if (vi)
-            for (int c = 0; c < 3; ++c)
-                if (fi[c] != 0.0) atomicAdd(acc + (size_t)c * n_pad + si, fi[c]);
+    typedef typename Vec<T>::type Vt;
+    extern __shared__ __align__(16) unsigned char raw[];
+    constexpr int ROWS = AP_CHUNK + 1;
+    T4 *sp = reinterpret_cast<T4 *>(raw);
+    T *se = reinterpret_cast<T *>(sp + ROWS), *ss = se + ROWS;
+    int *sl = reinterpret_cast<int *>(ss + ROWS);
+    const Layout<T, 1> ly;
+    constexpr int W = Vec<T>::W;
+    const int tid = threadIdx.x, s0 = ly.slot();
+    const Cands cs(la, ly.I);
+    Targets<T> tg;
+    tg.load(posw, s0, ly.h, n, rc * rc, T(1));
+    T ei[W], sgi[W];
+    for (int h = 0; h < W; ++h) {
+        ei[h] = s0 + h < n ? (T)lj[2 * perm[s0 + h]] : T(0);
+        sgi[h] = s0 + h < n ? (T)lj[2 * perm[s0 + h] + 1] : T(1);
     }
+    double e_sum = 0.0, fi[W][3] = {};
+    const int t0 = la.tile_off[ly.I], chunks = cs.chunks(), per = chunks ? (cs.n + chunks - 1) / chunks : 0;
+    const unsigned *list = la.list + list_entry_base(t0, ly.I, la.mult) / 2;
+    const uint2 *meta = la.meta + list_meta_base(t0, ly.I, la.mult) * 16 + ly.p;
+    const T4 *cpos = (const T4 *)la.cand_pos;
+    for (int c = 0; c < chunks; ++c) {
+        const int k0 = c * per, kc = min(per, cs.n - k0);
+        if (c) __syncthreads();
+        for (int k = tid; k < kc; k += 128) {
+            const size_t at = cs.at(k0 + k);
+            const int j = la.cand_j[at] & ~AP_CAND_SELF;
+            sp[k] = cpos[at];
+            se[k] = (T)lj[2 * perm[j]];
+            ss[k] = (T)lj[2 * perm[j] + 1];
+            sl[k] = j;
+        }
+        if (tid == 0) {
+            sp[kc] = phantom_pos<T>();
+            se[kc] = T(0);
+            ss[kc] = T(1);
+            sl[kc] = -1;
+        }
+        const uint2 m = meta[(size_t)c * 16];
+        __syncthreads();
+        auto side = [&](unsigned e) {
+            const int k = (e & 0xfff0u) >> 4, sj = sl[k];
+            const T ej = se[k];
+            if (!(ej > T(0)) || sj <= s0) return;
+            Vt R[3], pen;
+            bool exa, exb;
+            tg.template vector<true>(sp[k], e, R, pen, exa, exb);
+            for (int h = 0; h < W; ++h) {
+                const bool excluded = W == 2 ? (e >> h) & 1u : (e >> ly.h) & 1u;
+                if (Vec<T>::get(pen, h) < T(0) || excluded || sj <= s0 + h || !(ei[h] > T(0))) continue;
+                // the pair function in FP64 (few pairs: oxygens only): the force-shifted terms of
+                // close and far pairs cancel in the sum, which FP32 would resolve to ~1e-5 only
+                const double dx = Vec<T>::get(R[0], h), dy = Vec<T>::get(R[1], h), dz = Vec<T>::get(R[2], h);
+                double V, fr;
+                lj_fs<double>(dx * dx + dy * dy + dz * dz, sqrt((double)ei[h] * (double)ej),
+                              0.5 * ((double)sgi[h] + (double)ss[k]), (double)rc, V, fr);
+                e_sum += V;
+                const double f3[3] = {fr * dx, fr * dy, fr * dz};
+                for (int d = 0; d < 3; ++d) {
+                    fi[h][d] += f3[d];
+                    atomicAdd(acc + (size_t)d * n_pad + sj, -f3[d]);
+                }
+            }
+        };
+        walk(list + m.x / 2, meta_words(m), 0, ly.first, ly.STRIDE, side, side);
+    }
+    for (int h = 0; h < W; ++h)
+        for (int d = 0; d < 3; ++d) {
+            double v = fi[h][d];
+            for (int off = W == 2 ? 1 : 2; off < ly.TP; off <<= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (ly.first == 0 && v != 0.0) atomicAdd(acc + (size_t)d * n_pad + s0 + h, v);
+        }
     for (int off = 16; off; off >>= 1) e_sum += __shfl_xor_sync(0xffffffffu, e_sum, off);
-    if (lane == 0 && e_sum != 0.0) atomicAdd(energy, e_sum);
+    if ((tid & 31) == 0 && e_sum != 0.0) atomicAdd(energy, e_sum);
 }
 
 // out[i] (caller order) += acc[slot of i]
@@ -253,9 +257,9 @@ int lj_t(ap_ctx *ctx, const double *d_lj, double *d_energy, double *d_forces) {
     double *acc = ctx->qv;   // scratch [3][n_pad] (the PCG's q vector, free between solves)
     AP_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * ctx->n_pad, s));
     AP_CUDA(cudaMemsetAsync(d_energy, 0, sizeof(double), s));
-    auto kern = ctx->minimg ? k_lj_forces<T, true> : k_lj_forces<T, false>;
-    kern<<<4 * ctx->sm_count, 128, 0, s>>>(work_args(ctx), (const T4 *)ctx->posq, ctx->perm, d_lj, ctx->n, ctx->n_pad,
-                                          (T)P.cutoff, (T)P.box[0], (T)P.box[1], (T)P.box[2], acc, d_energy);
+    const size_t bytes = (size_t)(AP_CHUNK + 1) * (sizeof(T4) + 2 * sizeof(T) + sizeof(int));
+    AP_CUDA(allow_smem(k_lj_forces<T>, bytes));
+    k_lj_forces<T><<<ctx->n_blocks, 128, bytes, s>>>(list_args(ctx), (const T4 *)ctx->posw, ctx->perm, d_lj, ctx->n, ctx->n_pad, (T)P.cutoff, acc, d_energy);
     AP_CUDA(cudaGetLastError());
     k_add_unsort3<<<ap_grid_for(ctx->n, 256), 256, 0, s>>>(acc, ctx->iperm, ctx->n, ctx->n_pad, d_forces);
     AP_CUDA(cudaGetLastError());

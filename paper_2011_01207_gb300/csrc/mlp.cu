@@ -524,7 +524,6 @@ int features_slots(ap_ctx *ctx) {
         k_alpha_field<double><<<ap_grid_for(ctx->n_pad, 256), 256, 0, st>>>(ctx->E, ctx->alpha, ctx->n_pad, (dvec4 *)ctx->p);
     else
         k_alpha_field<float><<<ap_grid_for(ctx->n_pad, 256), 256, 0, st>>>(ctx->E, ctx->alpha, ctx->n_pad, (float4 *)ctx->p);
-    AP_CUDA(cudaMemsetAsync(ctx->e1s, 0, sizeof(double) * 3 * ctx->n_pad, st));
     int r = short_matvec_launch(ctx, ctx->p, ctx->e1s, st);
     if (r) return r;
     if (ctx->prec == AP_FP64)

@@ -11,8 +11,10 @@
 // GB300 choices (differences from the paper): cells are 1/4 of a 32-atom cube along x
 // and the cell order snakes through x and y, so every run of 32 atoms stays compact
 // without the paper's iterative refinement; the block-pair test is a brute-force
-// bounding-box sweep over block pairs (n_blocks^2 / 2 tests, a few ms even at 10^6
-// atoms), which needs no bit matrix at all.
+// bounding-box sweep over block pairs (n_blocks^2 tests, about a ms at 10^6 atoms),
+// which needs no bit matrix at all. Block pairs are kept in both orders: the pair lists made
+// from them (lists.cu) are per target atom. A rebuild with capacities that still hold allocates
+// nothing and reads its results back once.
 #include "common.cuh"
 
 #include <algorithm>
@@ -32,7 +34,9 @@ __device__ __forceinline__ double wrap1(double x, double L) {
     return (w >= L) ? 0.0 : w;
 }
 
-__global__ void k_cell_key(const double *__restrict__ xyz, int n, CellGrid g, int *__restrict__ key) {
+// cell of every atom, and the cells' counts
+__global__ void k_cell_key(const double *__restrict__ xyz, int n, CellGrid g, int *__restrict__ key,
+                           int *__restrict__ count) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double x = wrap1(xyz[3 * i + 0], g.lx), y = wrap1(xyz[3 * i + 1], g.ly), z = wrap1(xyz[3 * i + 2], g.lz);
@@ -45,14 +49,11 @@ __global__ void k_cell_key(const double *__restrict__ xyz, int n, CellGrid g, in
     int row = cz * g.ny + cyy;
     int cxx = (row & 1) ? (g.nx - 1 - cx) : cx;
     key[i] = row * g.nx + cxx;
+    atomicAdd(&count[key[i]], 1);
 }
 
-__global__ void k_histogram(const int *__restrict__ key, int n, int *__restrict__ count) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(&count[key[i]], 1);
-}
-
-// exclusive scan of m ints with one block of 1024 threads (build-time only)
+// exclusive scan of m ints with one block of 1024 threads (build-time only); with total given,
+// the sum also to it and to out[m]
 __global__ void k_scan_single(const int *__restrict__ in, int *__restrict__ out, int m, int *__restrict__ total) {
     __shared__ int sums[1024];
     int t = threadIdx.x;
@@ -74,7 +75,7 @@ __global__ void k_scan_single(const int *__restrict__ in, int *__restrict__ out,
         out[k] = run;
         run += v;
     }
-    if (t == 1023 && total) *total = sums[1023];
+    if (t == 1023 && total) *total = out[m] = sums[1023];
 }
 
 __global__ void k_scatter(const int *__restrict__ key, int n, const int *__restrict__ start,
@@ -99,15 +100,69 @@ __global__ void k_sort_cells(const int *__restrict__ start, const int *__restric
     }
 }
 
-__global__ void k_finish_perm(int *__restrict__ perm, int n, int n_pad, int *__restrict__ iperm) {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n_pad) return;
-    if (s >= n) { perm[s] = -1; return; }
-    iperm[perm[s]] = s;
+__global__ void k_pad_perm(int *__restrict__ perm, int n, int n_pad) {
+    const int s = n + threadIdx.x;
+    if (s < n_pad) perm[s] = -1;
 }
 
-// one warp per block: bounding box of its atoms (wrapped coordinates)
-__global__ void k_block_bbox(const double *__restrict__ xyz, const int *__restrict__ perm, int nb,
+// One warp per block: its atoms put in an order in which slots 2 k and 2 k + 1 hold near neighbours.
+// The pair kernels give a thread two such slots and walk one list for both, so a list is the
+// shorter the more of the two atoms' neighbours are the same: in water 175 entries per pair at
+// r_c = 7 A against 187 in the order of the cells. Greedy matching: every unmatched atom finds its
+// nearest unmatched one, mutual choices are matched, and so on (each round matches at least
+// the closest pair; distance ties go to the lower lane).
+__global__ void k_pair_order(const double *__restrict__ xyz, int nb, double3 L, int *__restrict__ perm) {
+    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (b >= nb) return;
+    const int a = perm[b * 32 + lane], a0 = perm[b * 32];
+    float x = 0.f, y = 0.f, z = 0.f;
+    if (a >= 0) {   // image nearest the block's first atom
+        const double d[3] = {xyz[3 * a] - xyz[3 * a0], xyz[3 * a + 1] - xyz[3 * a0 + 1], xyz[3 * a + 2] - xyz[3 * a0 + 2]};
+        x = (float)(d[0] - L.x * rint(d[0] / L.x));
+        y = (float)(d[1] - L.y * rint(d[1] / L.y));
+        z = (float)(d[2] - L.z * rint(d[2] / L.z));
+    }
+    const unsigned real = __ballot_sync(0xffffffffu, a >= 0);
+    unsigned open = real, leaders = 0u;
+    int partner = -1;
+    for (int round = 0; round < 16 && __popc(open) > 1; ++round) {
+        float best = 3e38f;
+        int nn = -1;
+        for (int j = 0; j < 32; ++j) {
+            const float dx = x - __shfl_sync(0xffffffffu, x, j), dy = y - __shfl_sync(0xffffffffu, y, j),
+                        dz = z - __shfl_sync(0xffffffffu, z, j), d = dx * dx + dy * dy + dz * dz;
+            if (((open >> j) & 1u) && j != lane && d < best) {
+                best = d;
+                nn = j;
+            }
+        }
+        if (!((open >> lane) & 1u)) nn = -1;
+        const int back = __shfl_sync(0xffffffffu, nn, nn < 0 ? lane : nn);
+        const bool mutual = nn >= 0 && back == lane;
+        if (mutual) partner = nn;
+        const unsigned done = __ballot_sync(0xffffffffu, mutual);
+        if (!done) break;   // only with coordinates that are not numbers
+        leaders |= __ballot_sync(0xffffffffu, mutual && lane < nn);
+        open &= ~done;
+    }
+    // pairs by their first lane, then the atoms left over, then the padding
+    const unsigned below = (1u << lane) - 1u;
+    const int pairs = __popc(leaders);
+    int slot;
+    if (partner >= 0) {
+        const int lead = min(lane, partner);
+        slot = 2 * __popc(leaders & ((1u << lead) - 1u)) + (lane > partner);
+    } else if (a >= 0) {
+        slot = 2 * pairs + __popc(open & below);
+    } else {
+        slot = 2 * pairs + __popc(open) + __popc(~real & below);
+    }
+    __syncwarp();
+    perm[b * 32 + slot] = a;
+}
+
+// one warp per block: bounding box of its atoms (wrapped coordinates); also the inverse order
+__global__ void k_block_bbox(const double *__restrict__ xyz, const int *__restrict__ perm, int nb, int *__restrict__ iperm,
                              double lx, double ly, double lz, float4 *__restrict__ center,
                              float4 *__restrict__ half, unsigned *__restrict__ hmax_bits) {
     int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -116,6 +171,7 @@ __global__ void k_block_bbox(const double *__restrict__ xyz, const int *__restri
     int a = perm[w * 32 + lane];
     double lo[3] = {1e300, 1e300, 1e300}, hi[3] = {-1e300, -1e300, -1e300};
     if (a >= 0) {
+        iperm[a] = w * 32 + lane;
         double p[3] = {wrap1(xyz[3 * a], lx), wrap1(xyz[3 * a + 1], ly), wrap1(xyz[3 * a + 2], lz)};
         for (int d = 0; d < 3; ++d) lo[d] = hi[d] = p[d];
     }
@@ -145,34 +201,40 @@ __device__ __forceinline__ bool blocks_near(float4 ci, float4 hi, float4 cj, flo
     return gx * gx + gy * gy + gz * gz < r2;
 }
 
-// one warp per block I: count (fill == nullptr) or write its partners J >= I
+// one warp per block I: count (tiles == nullptr) or write its partners J, I among them (as many as
+// fit: the caller looks at the total and grows the arrays)
 __global__ void k_tiles(const float4 *__restrict__ center, const float4 *__restrict__ half, int nb,
                         float3 L, float r2, int *__restrict__ count, const int *__restrict__ off,
-                        int2 *__restrict__ tiles, float4 *__restrict__ tshift, float4 *__restrict__ tshift_lo,
-                        double3 Ld) {
+                        TileRec *__restrict__ tiles, int cap, double3 Ld) {
     int I = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (I >= nb) return;
     float4 ci = center[I], hi = half[I];
     int pos = tiles ? off[I] : 0;
     int cnt = 0;
-    for (int base = I; base < nb; base += 32) {
+    for (int base = 0; base < nb; base += 32) {
         int J = base + lane;
         bool hit = false;
         if (J < nb) hit = blocks_near(ci, hi, center[J], half[J], L, r2);
         unsigned m = __ballot_sync(0xffffffffu, hit);
-        if (tiles && hit) {
-            int k = pos + __popc(m & ((1u << lane) - 1u));
-            tiles[k] = make_int2(I, J);
-            float4 cj = center[J];
+        const int k = pos + __popc(m & ((1u << lane) - 1u));
+        if (tiles && hit && k < cap) {
+            const float4 cj = center[J];
             // origin of J's image next to I, relative to I's origin: c_J - c_I + L k in FP64,
             // split into float hi + lo (the centres are the blocks' position origins)
             const double ox = (double)cj.x - (double)ci.x + Ld.x * rintf((ci.x - cj.x) / L.x);
             const double oy = (double)cj.y - (double)ci.y + Ld.y * rintf((ci.y - cj.y) / L.y);
             const double oz = (double)cj.z - (double)ci.z + Ld.z * rintf((ci.z - cj.z) / L.z);
-            const float hx = (float)ox, hy = (float)oy, hz = (float)oz;
-            tshift[k] = make_float4(hx, hy, hz, 0.f);
-            tshift_lo[k] = make_float4((float)(ox - hx), (float)(oy - hy), (float)(oz - hz), 0.f);
+            TileRec r;
+            r.J = J;
+            r.excl = -1;
+            r.hx = (float)ox;
+            r.hy = (float)oy;
+            r.hz = (float)oz;
+            r.lx = (float)(ox - r.hx);
+            r.ly = (float)(oy - r.hy);
+            r.lz = (float)(oz - r.hz);
+            tiles[k] = r;
         }
         pos += __popc(m);
         cnt += __popc(m);
@@ -180,54 +242,67 @@ __global__ void k_tiles(const float4 *__restrict__ center, const float4 *__restr
     if (!tiles && lane == 0) count[I] = cnt;
 }
 
-__device__ int find_tile(const int2 *__restrict__ tiles, int b, int e, int J) {
+__device__ int find_tile(const TileRec *__restrict__ tiles, int b, int e, int J) {
     while (b < e) {
         int m = (b + e) >> 1;
-        int v = tiles[m].y;
+        int v = tiles[m].J;
         if (v == J) return m;
         if (v < J) b = m + 1; else e = m;
     }
     return -1;
 }
 
-// pass 0: flag tiles holding excluded pairs; pass 1: set the mask bits
+// what a build reads back: tiles, whether an excluded pair lies outside them, exclusion slots, those
+// of diagonal tiles, and the blocks' largest half extents (float bits)
+enum { NB_TILES, NB_FAR, NB_SLOTS, NB_DIAG, NB_HMAX };
+
+// Exclusion masks of the tiles, word j-lane of tile (I, J) holding the excluded i-lanes, for both
+// orders of every pair. pass 0: flag the tiles (-2, diagonal ones -3); pass 1: set the mask bits.
 __global__ void k_excl(const int *__restrict__ off, const int *__restrict__ atoms, int n,
-                       const int *__restrict__ iperm, const int2 *__restrict__ tiles,
-                       const int *__restrict__ tile_off, int *__restrict__ tile_flag,
-                       const int *__restrict__ tile_excl, unsigned *__restrict__ masks,
-                       int pass, int *__restrict__ err) {
+                       const int *__restrict__ iperm, TileRec *__restrict__ tiles, int cap,
+                       const int *__restrict__ tile_off, unsigned *__restrict__ masks, int cap_slots, int pass,
+                       int *__restrict__ info) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+    if (i >= n || info[NB_TILES] > cap) return;
     for (int k = off[i]; k < off[i + 1]; ++k) {
         int j = atoms[k];
         if (j == i || j < 0 || j >= n) continue;
-        int si = iperm[i], sj = iperm[j];
-        int bI = si >> 5, li = si & 31, bJ = sj >> 5, lj = sj & 31;
-        if (bI > bJ) { int t = bI; bI = bJ; bJ = t; t = li; li = lj; lj = t; }
-        int t = find_tile(tiles, tile_off[bI], tile_off[bI + 1], bJ);
-        if (t < 0) { atomicExch(err, 1); continue; }
-        if (pass == 0) {
-            tile_flag[t] = 1;
-        } else {
-            unsigned *m = masks + (size_t)tile_excl[t] * 32;
-            atomicOr(&m[li], 1u << lj);
-            if (bI == bJ) atomicOr(&m[lj], 1u << li);
+        const int s[2] = {iperm[i], iperm[j]};
+        for (int d = 0; d < 2; ++d) {
+            const int bI = s[d] >> 5, li = s[d] & 31, bJ = s[1 - d] >> 5, lj = s[1 - d] & 31;
+            const int t = find_tile(tiles, tile_off[bI], tile_off[bI + 1], bJ);
+            if (t < 0) { atomicExch(info + NB_FAR, 1); continue; }
+            if (pass == 0) {
+                tiles[t].excl = bI == bJ ? -3 : -2;
+            } else {
+                const int e = tiles[t].excl;
+                if (e >= 0 && e < cap_slots) atomicOr(&masks[(size_t)e * 32 + lj], 1u << li);
+            }
         }
     }
 }
 
-__global__ void k_assign_slots(const int *__restrict__ flag, const int *__restrict__ scan, int m,
-                               int *__restrict__ tile_excl) {
+// a slot (in any order) and a cleared mask for every flagged tile
+__global__ void k_assign_slots(TileRec *__restrict__ tiles, int cap, unsigned *__restrict__ masks, int cap_slots,
+                               int *__restrict__ info) {
     int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < m) tile_excl[t] = flag[t] ? scan[t] : -1;
+    if (info[NB_TILES] > cap || t >= info[NB_TILES] || tiles[t].excl > -2) return;
+    const int e = atomicAdd(info + NB_SLOTS, 1);
+    if (tiles[t].excl == -3) atomicAdd(info + NB_DIAG, 1);
+    tiles[t].excl = e;
+    if (e < cap_slots)
+        for (int k = 0; k < 32; ++k) masks[(size_t)e * 32 + k] = 0u;
 }
 
+// room for `need` elements; `moved` is set when the array is allocated anew
 template <class P>
-int grow(ap_ctx *ctx, P **ptr, int *cap, long need, size_t elem) {
+int grow(ap_ctx *ctx, P **ptr, int *cap, long need, size_t elem, bool *moved = nullptr) {
     if (need <= *cap) return AP_OK;
     long c = std::max<long>(need + need / 4 + 64, 1024);
     if (*ptr) AP_CUDA(cudaFree(*ptr));
     *ptr = nullptr;
+    *cap = 0;
+    if (moved) *moved = true;
     AP_CUDA(cudaMalloc((void **)ptr, (size_t)c * elem));
     *cap = (int)c;
     return AP_OK;
@@ -252,108 +327,97 @@ int nb_build(ap_ctx *ctx, const double *d_xyz, const int *d_off, const int *d_at
 
     int r;
     if ((r = grow(ctx, &ctx->cell_count, &ctx->cap_cells, 3 * ncell + 3, sizeof(int)))) return r;
-    if ((r = grow(ctx, &ctx->tmp_int, &ctx->cap_tmp, std::max<long>(n, 4L * nb + 8), sizeof(int)))) return r;
-    int *count = ctx->cell_count, *start = count + ncell, *cursor = start + ncell;
-    int *key = ctx->tmp_int;
+    if ((r = grow(ctx, &ctx->tmp_int, &ctx->cap_tmp, std::max<long>(n, nb), sizeof(int)))) return r;
+    // the order, the tiles and the lists change from here on: none are valid until all are done
+    ctx->lists_valid = 0;
+    ctx->config_valid = 0;
+    int *count = ctx->cell_count, *cursor = count + ncell, *start = cursor + ncell;
+    int *key = ctx->tmp_int, *info = ctx->nb_info;
     const int T = 256;
 
-    AP_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * ncell, s));
-    AP_CUDA(cudaMemsetAsync(cursor, 0, sizeof(int) * ncell, s));
-    k_cell_key<<<ap_grid_for(n, T), T, 0, s>>>(d_xyz, n, g, key);
-    k_histogram<<<ap_grid_for(n, T), T, 0, s>>>(key, n, count);
+    AP_CUDA(cudaMemsetAsync(info, 0, sizeof(int) * 8, s));
+    AP_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * 2 * ncell, s));   // and the cursors
+    k_cell_key<<<ap_grid_for(n, T), T, 0, s>>>(d_xyz, n, g, key, count);
     k_scan_single<<<1, 1024, 0, s>>>(count, start, (int)ncell, nullptr);
     k_scatter<<<ap_grid_for(n, T), T, 0, s>>>(key, n, start, cursor, ctx->perm);
     k_sort_cells<<<ap_grid_for(ncell, T), T, 0, s>>>(start, count, (int)ncell, ctx->perm);
-    k_finish_perm<<<ap_grid_for(n_pad, T), T, 0, s>>>(ctx->perm, n, n_pad, ctx->iperm);
+    const double3 Ld = make_double3(P.box[0], P.box[1], P.box[2]);
+    if (n_pad > n) k_pad_perm<<<1, 32, 0, s>>>(ctx->perm, n, n_pad);
+    k_pair_order<<<ap_grid_for((long)nb * 32, T), T, 0, s>>>(d_xyz, nb, Ld, ctx->perm);
+    k_block_bbox<<<ap_grid_for((long)nb * 32, T), T, 0, s>>>(d_xyz, ctx->perm, nb, ctx->iperm, P.box[0], P.box[1], P.box[2],
+                                                           ctx->bcenter, ctx->bhalf, (unsigned *)(info + NB_HMAX));
     AP_CUDA(cudaGetLastError());
-
-    // block boxes
-    float4 *half = nullptr;
-    unsigned *hmax = nullptr;
-    AP_CUDA(cudaMallocAsync((void **)&half, sizeof(float4) * nb + 16, s));
-    AP_CUDA(cudaMallocAsync((void **)&hmax, sizeof(unsigned) * 4, s));
-    AP_CUDA(cudaMemsetAsync(hmax, 0, sizeof(unsigned) * 4, s));
-    k_block_bbox<<<ap_grid_for((long)nb * 32, T), T, 0, s>>>(d_xyz, ctx->perm, nb, P.box[0], P.box[1], P.box[2],
-                                                           ctx->bcenter, half, hmax);
-    float3 L = make_float3((float)P.box[0], (float)P.box[1], (float)P.box[2]);
-    float rl = (float)(P.cutoff + P.buffer);
+    const float3 L = make_float3((float)P.box[0], (float)P.box[1], (float)P.box[2]);
+    const float rl = (float)(P.cutoff + P.buffer);
     int *bcount = key;                 // reuse: key no longer needed
-    int *boff = key + nb + 1;
-    k_tiles<<<ap_grid_for((long)nb * 32, T), T, 0, s>>>(ctx->bcenter, half, nb, L, rl * rl, bcount, nullptr,
-                                                      nullptr, nullptr, nullptr, make_double3(P.box[0], P.box[1], P.box[2]));
-    int *d_total = boff + nb + 1;
-    k_scan_single<<<1, 1024, 0, s>>>(bcount, boff, nb, d_total);
-    int ntiles = 0;
-    unsigned hm[3];
-    AP_CUDA(cudaMemcpyAsync(&ntiles, d_total, sizeof(int), cudaMemcpyDeviceToHost, s));
-    AP_CUDA(cudaMemcpyAsync(hm, hmax, sizeof(unsigned) * 3, cudaMemcpyDeviceToHost, s));
-    AP_CUDA(cudaStreamSynchronize(s));
-    AP_CUDA(cudaMemcpyAsync(boff + nb, &ntiles, sizeof(int), cudaMemcpyHostToDevice, s));
-    if (ntiles <= 0) return ap_fail(ctx, AP_ERR_ARG, "no interacting blocks");
-
-    if ((r = grow(ctx, &ctx->tiles, &ctx->cap_tiles, ntiles, sizeof(int2)))) return r;
-    if (ctx->tshift) cudaFree(ctx->tshift);
-    if (ctx->tshift_lo) cudaFree(ctx->tshift_lo);
-    if (ctx->tile_excl) cudaFree(ctx->tile_excl);
-    AP_CUDA(cudaMalloc((void **)&ctx->tshift, sizeof(float4) * ctx->cap_tiles));
-    AP_CUDA(cudaMalloc((void **)&ctx->tshift_lo, sizeof(float4) * ctx->cap_tiles));
-    AP_CUDA(cudaMalloc((void **)&ctx->tile_excl, sizeof(int) * ctx->cap_tiles));
-    k_tiles<<<ap_grid_for((long)nb * 32, T), T, 0, s>>>(ctx->bcenter, half, nb, L, rl * rl, nullptr, boff,
-                                                      ctx->tiles, ctx->tshift, ctx->tshift_lo,
-                                                      make_double3(P.box[0], P.box[1], P.box[2]));
-    ctx->n_tiles = ntiles;
-    // keep the per-block tile offsets at the head of tmp_int for the exclusion pass
-    int *tile_off = boff;
-
-    // per-tile shift is exact when every dimension satisfies L > 2 r_c + 4 (h_max + buffer/2)
-    bool ok = true;
-    for (int d = 0; d < 3; ++d) {
-        float h;
-        memcpy(&h, &hm[d], sizeof(float));
-        if (!(P.box[d] > 2.0 * P.cutoff + 4.0 * (h + 0.5 * P.buffer))) ok = false;
-    }
-    ctx->minimg = ok ? 0 : 1;
-
-    // exclusion masks
-    ctx->n_excl_tiles = 0;
-    AP_CUDA(cudaMemsetAsync(ctx->tile_excl, 0xff, sizeof(int) * ntiles, s));
-    if (n_excl > 0) {
-        int *flag = nullptr, *scan = nullptr, *err = nullptr;
-        AP_CUDA(cudaMallocAsync((void **)&flag, sizeof(int) * (2L * ntiles + 4), s));
-        scan = flag + ntiles + 1;
-        AP_CUDA(cudaMallocAsync((void **)&err, sizeof(int) * 2, s));
-        AP_CUDA(cudaMemsetAsync(flag, 0, sizeof(int) * ntiles, s));
-        AP_CUDA(cudaMemsetAsync(err, 0, sizeof(int) * 2, s));
-        k_excl<<<ap_grid_for(n, T), T, 0, s>>>(d_off, d_atoms, n, ctx->iperm, ctx->tiles, tile_off, flag,
-                                              nullptr, nullptr, 0, err);
-        k_scan_single<<<1, 1024, 0, s>>>(flag, scan, ntiles, err + 1);
-        int hv[2];
-        AP_CUDA(cudaMemcpyAsync(hv, err, sizeof(int) * 2, cudaMemcpyDeviceToHost, s));
-        AP_CUDA(cudaStreamSynchronize(s));
-        if (hv[0]) {
-            cudaFreeAsync(flag, s); cudaFreeAsync(err, s); cudaFreeAsync(half, s); cudaFreeAsync(hmax, s);
-            return ap_fail(ctx, AP_ERR_ARG, "an excluded pair is farther apart than cutoff+buffer");
-        }
-        int nex = hv[1];
-        if ((r = grow(ctx, &ctx->excl_mask, &ctx->cap_excl, (long)nex * 32, sizeof(unsigned)))) return r;
-        k_assign_slots<<<ap_grid_for(ntiles, T), T, 0, s>>>(flag, scan, ntiles, ctx->tile_excl);
-        AP_CUDA(cudaMemsetAsync(ctx->excl_mask, 0, sizeof(unsigned) * 32 * (size_t)std::max(nex, 1), s));
-        k_excl<<<ap_grid_for(n, T), T, 0, s>>>(d_off, d_atoms, n, ctx->iperm, ctx->tiles, tile_off, flag,
-                                              ctx->tile_excl, ctx->excl_mask, 1, err);
-        ctx->n_excl_tiles = nex;
-        AP_CUDA(cudaFreeAsync(flag, s));
-        AP_CUDA(cudaFreeAsync(err, s));
-    }
-    AP_CUDA(cudaMemcpyAsync(ctx->tile_off, tile_off, sizeof(int) * (nb + 1), cudaMemcpyDeviceToDevice, s));
-    AP_CUDA(cudaFreeAsync(half, s));
-    AP_CUDA(cudaFreeAsync(hmax, s));
-    AP_CUDA(cudaStreamSynchronize(s));
+    const int warps = ap_grid_for((long)nb * 32, T);
+    k_tiles<<<warps, T, 0, s>>>(ctx->bcenter, ctx->bhalf, nb, L, rl * rl, bcount, nullptr, nullptr, 0, Ld);
+    k_scan_single<<<1, 1024, 0, s>>>(bcount, ctx->tile_off, nb, info + NB_TILES);
     AP_CUDA(cudaGetLastError());
-    if ((r = filter_alloc(ctx))) return r;
+
+    // Fill the tiles and their exclusion masks with the capacities of the last build, and read the
+    // counts back; where one did not hold, grow it and fill again (the first build of a context
+    // goes round twice or three times).
+    bool moved = false;
+    int h[8];
+    for (int round = 0;; ++round) {
+        if (ctx->cap_tiles > 0) {
+            k_tiles<<<warps, T, 0, s>>>(ctx->bcenter, ctx->bhalf, nb, L, rl * rl, nullptr, ctx->tile_off, ctx->tiles,
+                                        ctx->cap_tiles, Ld);
+            if (n_excl > 0) {
+                const int slots = ctx->cap_excl / 32;
+                AP_CUDA(cudaMemsetAsync(info + NB_FAR, 0, sizeof(int) * 3, s));
+                k_excl<<<ap_grid_for(n, T), T, 0, s>>>(d_off, d_atoms, n, ctx->iperm, ctx->tiles, ctx->cap_tiles,
+                                                      ctx->tile_off, ctx->excl_mask, slots, 0, info);
+                k_assign_slots<<<ap_grid_for(ctx->cap_tiles, T), T, 0, s>>>(ctx->tiles, ctx->cap_tiles, ctx->excl_mask,
+                                                                           slots, info);
+                k_excl<<<ap_grid_for(n, T), T, 0, s>>>(d_off, d_atoms, n, ctx->iperm, ctx->tiles, ctx->cap_tiles,
+                                                      ctx->tile_off, ctx->excl_mask, slots, 1, info);
+            }
+            AP_CUDA(cudaGetLastError());
+        }
+        AP_CUDA(cudaMemcpyAsync(h, info, sizeof(h), cudaMemcpyDeviceToHost, s));
+        AP_CUDA(cudaStreamSynchronize(s));
+        if (h[NB_TILES] <= 0) return ap_fail(ctx, AP_ERR_ARG, "no interacting blocks");
+        if (h[NB_TILES] > ctx->cap_tiles) {
+            if ((r = grow(ctx, &ctx->tiles, &ctx->cap_tiles, h[NB_TILES], sizeof(TileRec)))) return r;
+            continue;
+        }
+        if (h[NB_FAR]) return ap_fail(ctx, AP_ERR_ARG, "an excluded pair is farther apart than cutoff+buffer");
+        if ((long)h[NB_SLOTS] * 32 > ctx->cap_excl) {
+            if ((r = grow(ctx, &ctx->excl_mask, &ctx->cap_excl, (long)h[NB_SLOTS] * 32, sizeof(unsigned), &moved))) return r;
+            continue;
+        }
+        break;
+    }
+    ctx->n_tiles = h[NB_TILES];
+    ctx->n_excl_tiles = (h[NB_SLOTS] + h[NB_DIAG]) / 2;   // kept in both orders, diagonal ones once
+
+    // one image per tile is exact along every dimension with L > 2 r_c + 4 (h_max + buffer/2);
+    // along a shorter one an atom can be in range of a block in two
+    int dims = 0, mult = 1;
+    for (int d = 0; d < 3; ++d) {
+        float hm;
+        memcpy(&hm, &h[NB_HMAX + d], sizeof(float));
+        if (!(P.box[d] > 2.0 * P.cutoff + 4.0 * (hm + 0.5 * P.buffer))) {
+            dims |= 1 << d;
+            mult *= 2;
+        }
+    }
+    if (mult != ctx->list_mult) moved = true;
+    ctx->image_dims = dims;
+    ctx->list_mult = mult;
+    const long held = ctx->cap_lists;
+    if ((r = lists_alloc(ctx))) return r;
+    if (ctx->cap_lists != held) moved = true;
     ctx->lists_valid = 1;
-    ctx->config_valid = 0;
-    ctx->graph_ok = 0;             // pointers may have moved: rebuild the solve graph
-    ctx->graph_tried = 0;
-    if (ctx->solve_exec) { cudaGraphExecDestroy(ctx->solve_exec); ctx->solve_exec = nullptr; }
+    if (moved) {                   // captured solve loops hold the old pointers
+        ctx->graph_ok = 0;
+        ctx->graph_tried = 0;
+        if (ctx->solve_exec) cudaGraphExecDestroy(ctx->solve_exec);
+        ctx->solve_exec = nullptr;
+        diis_forget_graph(ctx);
+        dp_forget_graph(ctx);
+    }
     return AP_OK;
 }

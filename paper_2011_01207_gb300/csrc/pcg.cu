@@ -133,11 +133,11 @@ __device__ __forceinline__ bool last_block(unsigned int *counter) {
     return last;
 }
 
-// r_0 = E - A mu_0, partial sums of r.z and z.z; clears acc and p. The last block sums the
+// r_0 = E - A mu_0, partial sums of r.z and z.z; clears p. The last block sums the
 // partials in a fixed order and sets the initial state (eps_0, the stop decision).
 template <class T>
 __global__ void k_init_residual(const double *__restrict__ E, const double *__restrict__ alpha,
-                                const double *__restrict__ mu, double *__restrict__ acc,
+                                const double *__restrict__ mu, const double *__restrict__ acc,
                                 const T *__restrict__ rec, const double *__restrict__ dg, int n_pad,
                                 double *__restrict__ r, typename V4<T>::type *__restrict__ p,
                                 double *__restrict__ part, int fixed, PcgState *st, int n, double tol,
@@ -151,7 +151,6 @@ __global__ void k_init_residual(const double *__restrict__ E, const double *__re
             double Amu = a > 0.0 ? mu[k] * d - acc_value(acc, k, fixed) - (double)rec[k] : 0.0;
             double rr = a > 0.0 ? E[k] - Amu : 0.0;
             r[k] = rr;
-            acc[k] = 0.0;
             rz += rr * a * rr;
             zz += a * rr * a * rr;
         }
@@ -198,11 +197,11 @@ __global__ void k_direction(const double *__restrict__ r, const double *__restri
     p[s] = v;
 }
 
-// q = A p = (1/alpha - self) p - T_real p - T_rec p; partial p.q; clears acc. The last
+// q = A p = (1/alpha - self) p - T_real p - T_rec p; partial p.q. The last
 // block sums the partials and sets gamma = (r.z) / (p.q).
 template <class T>
 __global__ void k_apply(const typename V4<T>::type *__restrict__ p, const double *__restrict__ dg,
-                        double *__restrict__ acc, const T *__restrict__ rec, int n_pad, double *__restrict__ q,
+                        const double *__restrict__ acc, const T *__restrict__ rec, int n_pad, double *__restrict__ q,
                         double *__restrict__ part, PcgState *st, int fixed) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     double pq = 0.0, dummy = 0.0;
@@ -214,7 +213,6 @@ __global__ void k_apply(const typename V4<T>::type *__restrict__ p, const double
             const int k = c * n_pad + s;
             const double qq = pv[c] * d - acc_value(acc, k, fixed) - (double)rec[k];
             q[k] = qq;
-            acc[k] = 0.0;
             pq += pv[c] * qq;
         }
     }
@@ -298,9 +296,9 @@ __global__ void k_init_guess_f(const double *__restrict__ guess, const double *_
 }
 
 // r_0 = E - A mu_0 (formed in FP64 once per solve, stored in FP32), partial r.z and z.z of the
-// stored r; clears acc and p. The last block sets the initial state.
+// stored r; clears p. The last block sets the initial state.
 __global__ void k_init_residual_f(const double *__restrict__ E, const float2 *__restrict__ dga,
-                                  const float4 *__restrict__ mu, double *__restrict__ acc,
+                                  const float4 *__restrict__ mu, const double *__restrict__ acc,
                                   const float *__restrict__ rec, int n_pad, float4 *__restrict__ r,
                                   float4 *__restrict__ p, double *__restrict__ part, int fixed, PcgState *st, int n,
                                   double tol, int max_iter) {
@@ -315,7 +313,6 @@ __global__ void k_init_residual_f(const double *__restrict__ E, const float2 *__
             const int k = c * n_pad + s;
             const double Amu = d.y > 0.f ? (double)mv[c] * d.x - acc_value(acc, k, fixed) - (double)rec[k] : 0.0;
             rv[c] = d.y > 0.f ? (float)(E[k] - Amu) : 0.f;
-            acc[k] = 0.0;
             const float z = d.y * rv[c];
             f2_add_prod(rz, rv[c], z);
             f2_add_prod(zz, z, z);
@@ -349,22 +346,18 @@ __global__ void k_init_residual_f(const double *__restrict__ E, const float2 *__
     st->guard = 0;
 }
 
-// p = alpha r + beta p; clears the real-space accumulator and the PME grid for the next product
-// (here rather than in k_apply_f, whose last-block fence would wait for these stores, or as a
-// separate clearing step at the head of the reciprocal branch, which is the longer branch of
-// the product)
+// p = alpha r + beta p; clears the PME grid for the next product (here rather than in k_apply_f,
+// whose last-block fence would wait for these stores, or as a separate clearing step at the head
+// of the reciprocal branch)
 __global__ void k_direction_f(const float4 *__restrict__ r, const float2 *__restrict__ dga, int n_pad,
-                              float4 *__restrict__ p, const PcgState *__restrict__ st, double *__restrict__ acc,
-                              float *__restrict__ grid, size_t ngrid) {
+                              float4 *__restrict__ p, const PcgState *__restrict__ st, float *__restrict__ grid,
+                              size_t ngrid) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const size_t stride = (size_t)gridDim.x * blockDim.x;
     float4 *g4 = reinterpret_cast<float4 *>(grid);   // cudaMalloc'd: 16-byte aligned
     for (size_t i = s; i < ngrid / 4; i += stride) g4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (s < (int)(ngrid & 3)) grid[(ngrid & ~(size_t)3) + s] = 0.f;
     if (s >= n_pad) return;
-    acc[s] = 0.0;
-    acc[n_pad + s] = 0.0;
-    acc[2 * (size_t)n_pad + s] = 0.0;
     const float b = (float)st->beta, a = dga[s].y;
     const float4 rv = r[s];
     float4 v = p[s];
@@ -459,19 +452,23 @@ __global__ void k_unsort_f4(const float4 *__restrict__ src, const int *__restric
 // T p: reciprocal branch on `aux`, real space on `main`, joined back into `main`
 template <class T>
 int matvec_into(ap_ctx *ctx, const void *p, cudaStream_t main, cudaStream_t aux, bool grid_cleared = false) {
-    AP_CUDA(cudaEventRecord(ctx->ev_fork, main));
-    AP_CUDA(cudaStreamWaitEvent(aux, ctx->ev_fork, 0));
+    if (aux != main) {
+        AP_CUDA(cudaEventRecord(ctx->ev_fork, main));
+        AP_CUDA(cudaStreamWaitEvent(aux, ctx->ev_fork, 0));
+    }
     int rc = pme_dipole_field(ctx, p, aux, grid_cleared);
     if (rc) return rc;
     rc = real_matvec_launch(ctx, p, main);
     if (rc) return rc;
-    AP_CUDA(cudaEventRecord(ctx->ev_join, aux));
-    AP_CUDA(cudaStreamWaitEvent(main, ctx->ev_join, 0));
+    if (aux != main) {
+        AP_CUDA(cudaEventRecord(ctx->ev_join, aux));
+        AP_CUDA(cudaStreamWaitEvent(main, ctx->ev_join, 0));
+    }
     return AP_OK;
 }
 
 template <class T>
-int matvec_into(ap_ctx *ctx, const void *p) { return matvec_into<T>(ctx, p, ctx->s0, ctx->s1); }
+int matvec_into(ap_ctx *ctx, const void *p) { return matvec_into<T>(ctx, p, ctx->s0, aux_stream(ctx, ctx->s0, ctx->s1)); }
 
 double self_coef(const ap_ctx *ctx) { return 4.0 * std::pow(ctx->prm.ewald_beta, 3) / (3.0 * AP_SQRT_PI); }
 
@@ -482,7 +479,7 @@ int enqueue_iteration(ap_ctx *ctx, cudaGraphConditionalHandle h, int use_cond, c
     const int nb = ap_grid_for(ctx->n_pad, NT);
     double *part_pq = ctx->red_part, *part_rz = ctx->red_part + nb;
     if constexpr (std::is_same<T, float>::value) {
-        k_direction_f<<<nb, NT, 0, main>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st, ctx->acc,
+        k_direction_f<<<nb, NT, 0, main>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st,
                                            (float *)ctx->grid, ctx->ngrid);
         AP_CUDA(cudaGetLastError());
         int rc = matvec_into<T>(ctx, ctx->p, main, aux, true);   // the grid was cleared above
@@ -570,7 +567,6 @@ int solve_t(ap_ctx *ctx, const double *d_guess, double tol, int max_iter, double
     const int nb = ap_grid_for(ctx->n_pad, NT);
     cudaStream_t s = ctx->s0;
     AP_CUDA(cudaMemsetAsync(ctx->st, 0, sizeof(PcgState), s));
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, s));
     constexpr bool F32 = std::is_same<T, float>::value;   // FP32 vectors (mixed and fixed modes)
     if (F32)
         k_init_guess_f<<<nb, NT, 0, s>>>(d_guess, ctx->E, ctx->alpha, ctx->perm, ctx->n, ctx->n_pad, ctx->mu_f,
@@ -619,7 +615,7 @@ int solve_t(ap_ctx *ctx, const double *d_guess, double tol, int max_iter, double
         AP_CUDA(cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies));
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         AP_CUDA(cudaStreamBeginCaptureToGraph(ctx->s2, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-        rc = enqueue_iteration<T>(ctx, h, 1, ctx->s2, ctx->s3);
+        rc = enqueue_iteration<T>(ctx, h, 1, ctx->s2, aux_stream(ctx, ctx->s2, ctx->s3));
         cudaGraph_t captured = nullptr;
         cudaError_t ec = cudaStreamEndCapture(ctx->s2, &captured);
         if (rc) return rc;
@@ -684,7 +680,7 @@ int pcg_vectors_launch(ap_ctx *ctx, cudaStream_t s) {
         k_update<double><<<nb, NT, 0, s>>>((const T4 *)ctx->p, ctx->qv, ctx->alpha, ctx->n_pad, ctx->mu, ctx->r, ctx->st,
                                            part_rz, ctx->n, 0, 0);
     } else {
-        k_direction_f<<<nb, NT, 0, s>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st, ctx->acc,
+        k_direction_f<<<nb, NT, 0, s>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st,
                                         (float *)ctx->grid, ctx->ngrid);
         k_apply_f<<<nb, NT, 0, s>>>((const float4 *)ctx->p, ctx->dga_f, ctx->acc, (const float *)ctx->rec, ctx->n_pad,
                                     ctx->q_f, part_pq, ctx->st, ctx->fixed);
@@ -730,14 +726,12 @@ template <class T>
 int apply_t(ap_ctx *ctx, const double *d_v, double *d_out) {
     typedef typename V4<T>::type T4;
     const int nb = ap_grid_for(ctx->n_pad, NT);
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
     k_load_vec<T><<<nb, NT, 0, ctx->s0>>>(d_v, ctx->perm, ctx->n, ctx->n_pad, (T4 *)ctx->p);
     int rc = matvec_into<T>(ctx, ctx->p);
     if (rc) return rc;
     k_tp_out<T><<<nb, NT, 0, ctx->s0>>>((const T4 *)ctx->p, ctx->acc, (const T *)ctx->rec, self_coef(ctx),
                                          ctx->n_pad, ctx->qv, ctx->fixed);
     unsort3(ctx, ctx->qv, d_out, ctx->s0);
-    AP_CUDA(cudaMemsetAsync(ctx->acc, 0, sizeof(double) * 3 * ctx->n_pad, ctx->s0));
     AP_CUDA(cudaGetLastError());
     return AP_OK;
 }
