@@ -156,6 +156,8 @@ struct ap_ctx {
     void *grid2 = nullptr;    // second real grid (potential of the permanent multipoles, kept for forces)
     long long *grid_fx = nullptr;   // AP_FIXED: the spread's fixed-point grid (kept cleared)
     cufftHandle plan_r2c = 0, plan_c2r = 0;
+    float2 *fft_tw = nullptr;     // the library's own transforms (fft.cu): roots of the three sizes
+    float *fft_green = nullptr;   // and B C in their order; NULL where cuFFT is used
 
     // forces
     double *frc = nullptr;    // [3][n_pad] force accumulator (sorted)
@@ -221,6 +223,12 @@ int real_matvec_resident_per_sm(ap_ctx *ctx);
 int short_matvec_launch(ap_ctx *ctx, const void *p, double *out, cudaStream_t s);
 int real_forces_launch(ap_ctx *ctx, cudaStream_t s);
 int pme_init(ap_ctx *ctx);
+bool fft_supported(const ap_ctx *ctx);
+int fft_init(ap_ctx *ctx, const float *green);
+int fft_roundtrip_own(ap_ctx *ctx, const float *in, float2 *c, float *out, cudaStream_t s);
+int fft_there_own(ap_ctx *ctx, const float *in, float2 *c, cudaStream_t s);
+int fft_back_own(ap_ctx *ctx, float2 *c, float *out, cudaStream_t s);
+int2 fft_factors(const ap_ctx *ctx, int d);
 int pme_multipole_field(ap_ctx *ctx, cudaStream_t s);              // permanent: grid2 keeps phi_M
 // T_rec p -> rec; grid_cleared: the caller has zeroed the context's grid (no clearing here)
 int pme_dipole_field(ap_ctx *ctx, const void *p, cudaStream_t s, bool grid_cleared = false);

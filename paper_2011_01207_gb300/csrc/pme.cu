@@ -1,13 +1,14 @@
 // a3 / a6 - Smooth particle-mesh Ewald (paper Sec. 1.2.2, "Reciprocal space scheme": spread
 // the multipolar density with order-5 B-splines, forward FFT, product with the reciprocal
 // kernel, backward FFT, gather with B-spline derivatives; Fig. reci_scheme: atomics on
-// the grid). FFTs are cuFFT; spread, convolution and gather are the kernels below.
+// the grid). FFTs are the kernels of fft.cu, or cuFFT (FP64, large grids and other sizes); spread,
+// convolution and gather are the kernels below.
 //
 // Conventions (shared with the oracle by definition, not by code):
 //   u_a = K_a x_a / L_a, b = floor(u_a), w = u_a - b; stencil points k = (b - t) mod K_a,
 //   t = 0..4, weight M_5(w + t); a site spreads (q + d.grad + (1/3) Q:grad grad) of its
 //   weights, each Cartesian derivative being (K_a / L_a) d/du_a;
-//   phi_grid = C2R[ B(m) C(m) R2C[Q] ] (cuFFT's unnormalised inverse);
+//   phi_grid = C2R[ B(m) C(m) R2C[Q] ] (unnormalised inverse);
 //   C(m) = exp(-pi^2 |m|^2 / beta^2) / (pi V |m|^2), C(0) = 0, m aliased to [-K/2, K/2);
 //   B(m) = prod_a |b_a(m_a)|^2, |b(m)|^2 = 1/|sum_{k=0}^{3} M_5(k+1) e^{2 pi i m k / K}|^2,
 //   replaced by the mean of its neighbours where the sum vanishes (m = K/2).
@@ -503,6 +504,12 @@ int init_t(ap_ctx *ctx) {
     }
     AP_CUDA(cudaMemcpy(ctx->green, g.data(), sizeof(T) * g.size(), cudaMemcpyHostToDevice));
     bool dbl = sizeof(T) == 8;
+    if constexpr (std::is_same<T, float>::value) {
+        if (fft_supported(ctx)) {
+            const int r = fft_init(ctx, g.data());
+            if (r) return r;
+        }
+    }
     AP_CUFFT(cufftPlan3d(&ctx->plan_r2c, Kz, Ky, Kx, dbl ? CUFFT_D2Z : CUFFT_R2C));
     AP_CUFFT(cufftPlan3d(&ctx->plan_c2r, Kz, Ky, Kx, dbl ? CUFFT_Z2D : CUFFT_C2R));
     if (ctx->fixed) {
@@ -544,6 +551,8 @@ int gather_launch(ap_ctx *ctx, const T *phi, T *out, cudaStream_t s) {
 template <class T>
 int fft_roundtrip(ap_ctx *ctx, const PmeBufs &b, T *in, T *out, cudaStream_t s) {
     typedef typename FftTypes<T>::cplx C;
+    if constexpr (std::is_same<T, float>::value)
+        if (ctx->fft_green) return fft_roundtrip_own(ctx, in, (float2 *)b.cgrid, out, s);
     AP_CUFFT(cufftSetStream(b.r2c, s));
     AP_CUFFT(cufftSetStream(b.c2r, s));
     if (sizeof(T) == 8) {
@@ -643,15 +652,15 @@ int dipole_field_t(ap_ctx *ctx, const void *p, void *rec_out, const PmeBufs &bf,
 template <class T>
 __global__ void k_virial_sf(const typename FftTypes<T>::cplx *__restrict__ Fmu,
                             const typename FftTypes<T>::cplx *__restrict__ Phi, const T *__restrict__ green,
-                            int Kx, int Ky, int Kz, double iLx, double iLy, double iLz, double pib2,
+                            int Kx, int Ky, int Kz, int2 fy, int2 fz, double iLx, double iLy, double iLz, double pib2,
                             double inv_k3, double f, size_t m, double *__restrict__ acc, int fixed) {
     const size_t idx = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (idx < m) {
         const int hx = Kx / 2 + 1;
         const int ix = (int)(idx % hx);
-        const int iy = (int)((idx / hx) % Ky);
-        const int iz = (int)(idx / ((size_t)hx * Ky));
+        const int py = (int)((idx / hx) % Ky), pz = (int)(idx / ((size_t)hx * Ky));
+        const int iy = py / fy.y + fy.x * (py % fy.y), iz = pz / fz.y + fz.x * (pz % fz.y);   // fft_factors()
         const int kx = ix < (Kx + 1) / 2 ? ix : ix - Kx;
         const int ky = iy < (Ky + 1) / 2 ? iy : iy - Ky;
         const int kz = iz < (Kz + 1) / 2 ? iz : iz - Kz;
@@ -713,28 +722,40 @@ int forces_t(ap_ctx *ctx, const void *mu4, double *gbuf, int with_M, cudaStream_
         r = fft_roundtrip<T>(ctx, bf, (T *)ctx->grid, (T *)ctx->grid, s);
         if (r) return r;
     } else {
-        const bool dbl = sizeof(T) == 8;
+        // the transforms of the dipoles' grid and of the permanent potential, the structure-factor
+        // sum over them, then the rest of the round trip
+        const bool dbl = sizeof(T) == 8, own = ctx->fft_green != nullptr;
         AP_CUFFT(cufftSetStream(bf.r2c, s));
         AP_CUFFT(cufftSetStream(bf.c2r, s));
-        if (dbl) AP_CUFFT(cufftExecD2Z(bf.r2c, (cufftDoubleReal *)ctx->grid, (cufftDoubleComplex *)ctx->cgrid));
-        else AP_CUFFT(cufftExecR2C(bf.r2c, (cufftReal *)ctx->grid, (cufftComplex *)ctx->cgrid));
-        if (with_M) {
-            // the permanent potential, copied so that its grid stays untouched for later calls
-            AP_CUDA(cudaMemcpyAsync(ctx->grid, ctx->grid2, sizeof(T) * ctx->ngrid, cudaMemcpyDeviceToDevice, s));
-            if (dbl) AP_CUFFT(cufftExecD2Z(bf.r2c, (cufftDoubleReal *)ctx->grid, (cufftDoubleComplex *)ctx->cgrid_v));
-            else AP_CUFFT(cufftExecR2C(bf.r2c, (cufftReal *)ctx->grid, (cufftComplex *)ctx->cgrid_v));
+        if (own) {
+            if ((r = fft_there_own(ctx, (const float *)ctx->grid, (float2 *)ctx->cgrid, s))) return r;
+            if (with_M && (r = fft_there_own(ctx, (const float *)ctx->grid2, (float2 *)ctx->cgrid_v, s))) return r;
+        } else {
+            if (dbl) AP_CUFFT(cufftExecD2Z(bf.r2c, (cufftDoubleReal *)ctx->grid, (cufftDoubleComplex *)ctx->cgrid));
+            else AP_CUFFT(cufftExecR2C(bf.r2c, (cufftReal *)ctx->grid, (cufftComplex *)ctx->cgrid));
+            if (with_M) {
+                // the permanent potential, copied so that its grid stays untouched for later calls
+                AP_CUDA(cudaMemcpyAsync(ctx->grid, ctx->grid2, sizeof(T) * ctx->ngrid, cudaMemcpyDeviceToDevice, s));
+                if (dbl) AP_CUFFT(cufftExecD2Z(bf.r2c, (cufftDoubleReal *)ctx->grid, (cufftDoubleComplex *)ctx->cgrid_v));
+                else AP_CUFFT(cufftExecR2C(bf.r2c, (cufftReal *)ctx->grid, (cufftComplex *)ctx->cgrid_v));
+            }
         }
         const ap_params &P = ctx->prm;
         const double k3 = (double)ctx->K[0] * ctx->K[1] * ctx->K[2];
         k_virial_sf<T><<<ap_grid_for((long)ctx->ncgrid, 256), 256, 0, s>>>(
-            (const C *)ctx->cgrid, with_M ? (const C *)ctx->cgrid_v : nullptr, (const T *)ctx->green, ctx->K[0],
-            ctx->K[1], ctx->K[2], 1.0 / P.box[0], 1.0 / P.box[1], 1.0 / P.box[2],
+            (const C *)ctx->cgrid, with_M ? (const C *)ctx->cgrid_v : nullptr,
+            own ? (const T *)ctx->fft_green : (const T *)ctx->green, ctx->K[0], ctx->K[1], ctx->K[2], fft_factors(ctx, 1),
+            fft_factors(ctx, 2), 1.0 / P.box[0], 1.0 / P.box[1], 1.0 / P.box[2],
             M_PI * M_PI / (P.ewald_beta * P.ewald_beta), 1.0 / k3, AP_COULOMB, ctx->ncgrid, vir, ctx->fixed);
-        k_convolve<T><<<ap_grid_for((long)ctx->ncgrid, 256), 256, 0, s>>>((C *)ctx->cgrid, (const T *)ctx->green,
-                                                                         ctx->ncgrid);
-        AP_CUDA(cudaGetLastError());
-        if (dbl) AP_CUFFT(cufftExecZ2D(bf.c2r, (cufftDoubleComplex *)ctx->cgrid, (cufftDoubleReal *)ctx->grid));
-        else AP_CUFFT(cufftExecC2R(bf.c2r, (cufftComplex *)ctx->cgrid, (cufftReal *)ctx->grid));
+        if (own) {
+            if ((r = fft_back_own(ctx, (float2 *)ctx->cgrid, (float *)ctx->grid, s))) return r;
+        } else {
+            k_convolve<T><<<ap_grid_for((long)ctx->ncgrid, 256), 256, 0, s>>>((C *)ctx->cgrid, (const T *)ctx->green,
+                                                                             ctx->ncgrid);
+            AP_CUDA(cudaGetLastError());
+            if (dbl) AP_CUFFT(cufftExecZ2D(bf.c2r, (cufftDoubleComplex *)ctx->cgrid, (cufftDoubleReal *)ctx->grid));
+            else AP_CUFFT(cufftExecC2R(bf.c2r, (cufftComplex *)ctx->cgrid, (cufftReal *)ctx->grid));
+        }
     }
     k_gather_derivs<T><<<ap_grid_for(ctx->n, 128), 128, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, (const T *)ctx->grid,
                                                                gbuf, ctx->n_pad, 20, pc);
