@@ -18,9 +18,12 @@
 #include "common.cuh"
 #include "vec_f32.cuh"
 
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <cstdlib>
 #include <type_traits>
+#include <utility>
 
 void unsort3(ap_ctx *ctx, const double *src, double *out, cudaStream_t s);
 
@@ -438,6 +441,128 @@ __global__ void k_update_f(const float4 *__restrict__ p, const float4 *__restric
     if (threadIdx.x == 0) finish_iteration(st, rzn, zzt, n, h, use_cond);
 }
 
+// The vector work of one iteration in one kernel, for systems of up to 16,384 slots: apply, update and
+// the next direction, by one cluster of at most eight CTAs whose threads hold their slots' p, q and r in
+// registers throughout. The two dot products are summed over the cluster through its shared memory, in a
+// fixed order and alike in every CTA. On small systems the three kernels were bound by their launches and
+// by the chain store - fence - counter - last block, not by their arithmetic.
+namespace cg = cooperative_groups;
+constexpr int ST = 512, ST_CTAS = 8, ST_SLOTS = 4;   // threads, CTAs, slots per thread at most
+
+// the cluster's sums of a and b (thread 0's of each CTA) in every thread of warp 0
+__device__ __forceinline__ void cluster_sum2(const cg::cluster_group &cl, double (*mine)[2], double &a, double &b) {
+    if (threadIdx.x == 0) {
+        (*mine)[0] = a;
+        (*mine)[1] = b;
+    }
+    cl.sync();
+    if (threadIdx.x < 32) {
+        a = b = 0.0;
+        if (threadIdx.x < cl.num_blocks()) {
+            const double *o = cl.map_shared_rank(&(*mine)[0], threadIdx.x);
+            a = o[0];
+            b = o[1];
+        }
+        for (int off = ST_CTAS / 2; off; off >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, off);
+            b += __shfl_xor_sync(0xffffffffu, b, off);
+        }
+    }
+}
+
+template <int PER>
+__global__ void __launch_bounds__(ST) k_step_f(float4 *__restrict__ p, const float2 *__restrict__ dga,
+                                               const double *__restrict__ acc, const float *__restrict__ rec, int n_pad,
+                                               float4 *__restrict__ mu, float4 *__restrict__ r, PcgState *st, int fixed,
+                                               int n, cudaGraphConditionalHandle h, int use_cond,
+                                               float *__restrict__ grid, size_t ngrid) {
+    __shared__ double part[2][2];
+    __shared__ float scale[2];   // gamma, beta
+    const cg::cluster_group cl = cg::this_cluster();
+    const int s0 = blockIdx.x * ST + threadIdx.x, stride = gridDim.x * ST;
+    const double rz0 = st->rz;   // rewritten below, after the last of the cluster's barriers that sum
+    float4 pv[PER], rv[PER], mv[PER];
+    float qv[PER][3], al[PER];
+    F2 pq = {0.f, 0.f}, none = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int s = s0 + k * stride;
+        pv[k] = rv[k] = mv[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        qv[k][0] = qv[k][1] = qv[k][2] = al[k] = 0.f;
+        if (s < n_pad) {
+            const float2 d = dga[s];
+            pv[k] = p[s];
+            rv[k] = r[s];
+            mv[k] = mu[s];
+            al[k] = d.y;
+            const float v[3] = {pv[k].x, pv[k].y, pv[k].z};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const int at = c * n_pad + s;
+                qv[k][c] = fmaf(v[c], d.x, -acc_f32(acc, at, fixed)) - rec[at];
+                f2_add_prod(pq, v[c], qv[k][c]);
+            }
+        }
+    }
+    double a = 0.0, b = 0.0;
+    block_sum2_f2<ST>(pq, none, a, b);
+    cluster_sum2(cl, &part[0], a, b);
+    double gamma = 0.0;
+    if (threadIdx.x == 0) {
+        gamma = rz0 / a;
+        scale[0] = (float)gamma;
+        if (blockIdx.x == 0) {
+            st->pq = a;
+            st->gamma = gamma;
+        }
+    }
+    __syncthreads();
+    const float g = scale[0];
+    F2 rz = {0.f, 0.f}, zz = {0.f, 0.f};
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        mv[k].x = fmaf(g, pv[k].x, mv[k].x);
+        mv[k].y = fmaf(g, pv[k].y, mv[k].y);
+        mv[k].z = fmaf(g, pv[k].z, mv[k].z);
+        rv[k].x = fmaf(-g, qv[k][0], rv[k].x);
+        rv[k].y = fmaf(-g, qv[k][1], rv[k].y);
+        rv[k].z = fmaf(-g, qv[k][2], rv[k].z);
+        if (s0 + k * stride < n_pad) {
+            const float rr[3] = {rv[k].x, rv[k].y, rv[k].z};
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float z = al[k] * rr[c];
+                f2_add_prod(rz, rr[c], z);
+                f2_add_prod(zz, z, z);
+            }
+        }
+    }
+    a = b = 0.0;
+    block_sum2_f2<ST>(rz, zz, a, b);
+    cluster_sum2(cl, &part[1], a, b);
+    if (threadIdx.x == 0) scale[1] = (float)(a / rz0);
+    __syncthreads();
+    // no CTA leaves while another may still read its sums
+    auto token = cl.barrier_arrive();
+    const float be = scale[1];
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        const int s = s0 + k * stride;
+        if (s < n_pad) {
+            mu[s] = mv[k];
+            r[s] = rv[k];
+            p[s] = make_float4(fmaf(al[k], rv[k].x, be * pv[k].x), fmaf(al[k], rv[k].y, be * pv[k].y),
+                               fmaf(al[k], rv[k].z, be * pv[k].z), 0.f);
+        }
+    }
+    // the PME grid for the next product
+    float4 *g4 = reinterpret_cast<float4 *>(grid);
+    for (size_t i = s0; i < ngrid / 4; i += stride) g4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (s0 < (int)(ngrid & 3)) grid[(ngrid & ~(size_t)3) + s0] = 0.f;
+    if (blockIdx.x == 0 && threadIdx.x == 0) finish_iteration(st, a, b, n, h, use_cond);
+    cl.barrier_wait(std::move(token));
+}
+
 // the FP32 dipoles to the caller's order in FP64
 __global__ void k_unsort_f4(const float4 *__restrict__ src, const int *__restrict__ iperm, int n,
                             double *__restrict__ out) {
@@ -472,6 +597,41 @@ int matvec_into(ap_ctx *ctx, const void *p) { return matvec_into<T>(ctx, p, ctx-
 
 double self_coef(const ap_ctx *ctx) { return 4.0 * std::pow(ctx->prm.ewald_beta, 3) / (3.0 * AP_SQRT_PI); }
 
+// whether the vector work of an iteration is k_step_f; a solve then forms the first direction before
+// its loop, the kernel every further one
+// (the line is the cluster's capacity: one iteration in the graph 38.8 -> 32.8 us at 648 atoms, 41.0 -> 35.7 at
+// 3,009, 51.5 -> 50.3 at 12,288, where eight SMs' bandwidth begins to show)
+bool one_step(const ap_ctx *ctx) { return ctx->prec != AP_FP64 && ctx->n_pad <= ST * ST_CTAS * ST_SLOTS; }
+
+int direction_launch(ap_ctx *ctx, cudaStream_t s) {
+    k_direction_f<<<ap_grid_for(ctx->n_pad, NT), NT, 0, s>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st,
+                                                           (float *)ctx->grid, ctx->ngrid);
+    AP_CUDA(cudaGetLastError());
+    return AP_OK;
+}
+
+int step_launch(ap_ctx *ctx, cudaGraphConditionalHandle h, int use_cond, cudaStream_t s) {
+    auto launch = [&](auto kern, int per) {
+        cudaLaunchConfig_t cfg = {};
+        const int ctas = (ctx->n_pad + ST * per - 1) / (ST * per);
+        cfg.gridDim = dim3(ctas);
+        cfg.blockDim = dim3(ST);
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = ctas;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, kern, (float4 *)ctx->p, (const float2 *)ctx->dga_f, (const double *)ctx->acc,
+                                  (const float *)ctx->rec, ctx->n_pad, ctx->mu_f, ctx->r_f, ctx->st, ctx->fixed, ctx->n,
+                                  h, use_cond, (float *)ctx->grid, ctx->fixed ? (size_t)0 : ctx->ngrid);   // fixed: the conversion writes it whole
+    };
+    const int cap = ST * ST_CTAS;
+    AP_CUDA(ctx->n_pad <= cap ? launch(k_step_f<1>, 1) : ctx->n_pad <= 2 * cap ? launch(k_step_f<2>, 2) : launch(k_step_f<4>, 4));
+    return AP_OK;
+}
+
 template <class T>
 int enqueue_iteration(ap_ctx *ctx, cudaGraphConditionalHandle h, int use_cond, cudaStream_t main,
                       cudaStream_t aux) {
@@ -479,6 +639,10 @@ int enqueue_iteration(ap_ctx *ctx, cudaGraphConditionalHandle h, int use_cond, c
     const int nb = ap_grid_for(ctx->n_pad, NT);
     double *part_pq = ctx->red_part, *part_rz = ctx->red_part + nb;
     if constexpr (std::is_same<T, float>::value) {
+        if (one_step(ctx)) {
+            int rc = matvec_into<T>(ctx, ctx->p, main, aux, true);
+            return rc ? rc : step_launch(ctx, h, use_cond, main);
+        }
         k_direction_f<<<nb, NT, 0, main>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st,
                                            (float *)ctx->grid, ctx->ngrid);
         AP_CUDA(cudaGetLastError());
@@ -586,6 +750,7 @@ int solve_t(ap_ctx *ctx, const double *d_guess, double tol, int max_iter, double
                                               ctx->n_pad, ctx->r, (T4 *)ctx->p, ctx->red_part, ctx->fixed, ctx->st,
                                               ctx->n, tol, max_iter);
     AP_CUDA(cudaGetLastError());
+    if (one_step(ctx) && (rc = direction_launch(ctx, s))) return rc;
     // the solution to the caller's order, in FP64
     auto unsort_mu = [&](cudaStream_t st) {
         if (F32) k_unsort_f4<<<ap_grid_for(ctx->n, 256), 256, 0, st>>>(ctx->mu_f, ctx->iperm, ctx->n, d_mu);
@@ -679,6 +844,8 @@ int pcg_vectors_launch(ap_ctx *ctx, cudaStream_t s) {
                                           ctx->qv, part_pq, ctx->st, ctx->fixed);
         k_update<double><<<nb, NT, 0, s>>>((const T4 *)ctx->p, ctx->qv, ctx->alpha, ctx->n_pad, ctx->mu, ctx->r, ctx->st,
                                            part_rz, ctx->n, 0, 0);
+    } else if (one_step(ctx)) {
+        return step_launch(ctx, 0, 0, s);
     } else {
         k_direction_f<<<nb, NT, 0, s>>>(ctx->r_f, ctx->dga_f, ctx->n_pad, (float4 *)ctx->p, ctx->st,
                                         (float *)ctx->grid, ctx->ngrid);
