@@ -14,6 +14,7 @@
 //   replaced by the mean of its neighbours where the sum vanishes (m = K/2).
 // Grid layout: [z][y][x], x contiguous; complex half grid [z][y][x/2+1].
 #include "common.cuh"
+#include "pair_math.cuh"   // packed fma2
 
 #include <algorithm>
 #include <climits>
@@ -164,8 +165,72 @@ __global__ void k_convolve(typename FftTypes<T>::cplx *__restrict__ c, const T *
     c[i].y *= g;
 }
 
-// gather the field -grad(phi) at every atom ---------------------------------------------
-template <class T>
+// gathers --------------------------------------------------------------------------------
+// The stencil's five points of a grid row with their weights and derivatives along x; sums() gives
+// S[d] = sum_t (d-th derivative)_t row[k_t].
+template <class T, int ND, bool WIDE>
+struct RowX {
+    const Stencil<T> &st;
+    __device__ __forceinline__ RowX(const Stencil<T> &s, int) : st(s) {}
+    __device__ __forceinline__ void sums(const T *row, T *S) const {
+#pragma unroll
+        for (int d = 0; d < ND; ++d) S[d] = 0;
+#pragma unroll
+        for (int t = 0; t < 5; ++t) {
+            const T v = row[st.k[0][t]];
+            S[0] += st.th[0][t] * v;
+            S[1] += st.d1[0][t] * v;
+            if (ND > 2) S[2] += st.d2[0][t] * v;
+            if (ND > 3) S[3] += st.d3[0][t] * v;
+        }
+    }
+};
+// FP32 with Kx a multiple of four: the two aligned groups of four points that hold the five, two
+// loads a row instead of five (the gathers are bound by their load instructions), and weights moved by
+// the first point's place in its group, zero at the three points beside the stencil: field gather
+// 16.7 -> 14.2 us at 96,000 atoms, 158 -> 147 at 1,065,000. (Loads chosen per row by the alignment
+// diverge, and are slower than five scalar ones.)
+template <int ND>
+struct RowX<float, ND, true> {
+    float2 w[8][ND / 2];
+    int x0, x1;
+    __device__ __forceinline__ RowX(const Stencil<float> &s, int Kx) {
+        const int k = s.k[0][4], mis = k & 3;   // the first point along x is t = 4
+        x0 = k - mis;
+        x1 = x0 + 4 == Kx ? 0 : x0 + 4;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+#pragma unroll
+            for (int d = 0; d < ND / 2; ++d) w[j][d] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                if (j >= m && j - m <= 4 && mis == m) {
+                    const int t = 4 - (j - m);
+                    w[j][0] = make_float2(s.th[0][t], s.d1[0][t]);
+                    if (ND > 2) w[j][ND / 2 - 1] = make_float2(s.d2[0][t], s.d3[0][t]);
+                }
+        }
+    }
+    __device__ __forceinline__ void sums(const float *row, float *S) const {
+        const float4 a = *reinterpret_cast<const float4 *>(row + x0), b = *reinterpret_cast<const float4 *>(row + x1);
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        float2 q[ND / 2];
+#pragma unroll
+        for (int d = 0; d < ND / 2; ++d) q[d] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+#pragma unroll
+            for (int d = 0; d < ND / 2; ++d) q[d] = fma2(splat2(v[j]), w[j][d], q[d]);
+#pragma unroll
+        for (int d = 0; d < ND / 2; ++d) {
+            S[2 * d] = q[d].x;
+            S[2 * d + 1] = q[d].y;
+        }
+    }
+};
+
+// the field -grad(phi) at every atom
+template <class T, bool WIDE>
 __global__ void k_gather_field(const int4 *__restrict__ stb, const typename V4<T>::type *__restrict__ stw,
                                const T *__restrict__ phi, T *__restrict__ out, int n_pad, PmeConsts<T> pc) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -173,6 +238,7 @@ __global__ void k_gather_field(const int4 *__restrict__ stb, const typename V4<T
     Stencil<T> st;
     make_stencil<T, 1>(pc, stb[i], stw[i], st);
     const int Kx = pc.K[0], Ky = pc.K[1];
+    const RowX<T, 2, WIDE> rx(st, Kx);
     T gx = 0, gy = 0, gz = 0;
 #pragma unroll
     for (int t3 = 0; t3 < 5; ++t3) {
@@ -180,17 +246,11 @@ __global__ void k_gather_field(const int4 *__restrict__ stb, const typename V4<T
 #pragma unroll
         for (int t2 = 0; t2 < 5; ++t2) {
             const T y0 = st.th[1][t2], y1 = st.d1[1][t2];
-            const T *row = phi + ((size_t)st.k[2][t3] * Ky + st.k[1][t2]) * Kx;
-            T s0 = 0, s1 = 0;
-#pragma unroll
-            for (int t1 = 0; t1 < 5; ++t1) {
-                const T v = row[st.k[0][t1]];
-                s0 += st.th[0][t1] * v;
-                s1 += st.d1[0][t1] * v;
-            }
-            gx += s1 * y0 * z0;
-            gy += s0 * y1 * z0;
-            gz += s0 * y0 * z1;
+            T S[2];
+            rx.sums(phi + ((size_t)st.k[2][t3] * Ky + st.k[1][t2]) * Kx, S);
+            gx += S[1] * y0 * z0;
+            gy += S[0] * y1 * z0;
+            gz += S[0] * y0 * z1;
         }
     }
     out[i] = -gx * pc.s[0];
@@ -322,6 +382,38 @@ __device__ __forceinline__ void make_stencil_plane(const PmeConsts<T> &pc, int4 
     kz = k < 0 ? k + pc.K[2] : k;
 }
 
+// the field with five threads per atom, a z-plane each, summed over the five lanes
+template <class T, bool WIDE>
+__global__ void k_gather_field5(const int4 *__restrict__ stb, const typename V4<T>::type *__restrict__ stw,
+                                const T *__restrict__ phi, T *__restrict__ out, int n_pad, PmeConsts<T> pc) {
+    const Lane5 l = lane5(pc.n);
+    T g[3] = {0, 0, 0};
+    if (l.ok) {
+        Stencil<T> st;
+        int kz;
+        T z0, z1;
+        make_stencil_plane<T>(pc, stb[l.i], stw[l.i], l.t3, st, kz, z0, z1);
+        const int Kx = pc.K[0], Ky = pc.K[1];
+        const RowX<T, 2, WIDE> rx(st, Kx);
+#pragma unroll
+        for (int t2 = 0; t2 < 5; ++t2) {
+            const T y0 = st.th[1][t2], y1 = st.d1[1][t2];
+            T S[2];
+            rx.sums(phi + ((size_t)kz * Ky + st.k[1][t2]) * Kx, S);
+            g[0] += S[1] * y0 * z0;
+            g[1] += S[0] * y1 * z0;
+            g[2] += S[0] * y0 * z1;
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        T sum = g[c];
+#pragma unroll
+        for (int k = 1; k < 5; ++k) sum += __shfl_down_sync(0xffffffffu, g[c], k);
+        if (l.ok && l.t3 == 0) out[(size_t)c * n_pad + l.i] = -sum * pc.s[c];
+    }
+}
+
 template <class T, bool FX>
 __global__ void k_spread_dipoles5(const int4 *__restrict__ stb, const typename V4<T>::type *__restrict__ stw,
                                   const typename V4<T>::type *__restrict__ pv, void *__restrict__ grid,
@@ -385,7 +477,7 @@ __global__ void k_spread_multipoles5(const typename V4<T>::type *__restrict__ po
 // derivatives of phi up to third order (20 components) for the forces -------------------
 // component order: [0] phi; [1..3] x y z; [4..9] xx yy zz xy xz yz;
 // [10..19] xxx yyy zzz xxy xxz xyy yyz xzz yzz xyz
-template <class T>
+template <class T, bool WIDE>
 __global__ void k_gather_derivs(const int4 *__restrict__ stb, const typename V4<T>::type *__restrict__ stw,
                                 const T *__restrict__ phi, double *__restrict__ out, int n_pad, int ncomp,
                                 PmeConsts<T> pc) {
@@ -394,6 +486,7 @@ __global__ void k_gather_derivs(const int4 *__restrict__ stb, const typename V4<
     Stencil<T> st;
     make_stencil<T, 3>(pc, stb[i], stw[i], st);
     const int Kx = pc.K[0], Ky = pc.K[1];
+    const RowX<T, 4, WIDE> rx(st, Kx);
     T D[20];
 #pragma unroll
     for (int c = 0; c < 20; ++c) D[c] = 0;
@@ -403,16 +496,8 @@ __global__ void k_gather_derivs(const int4 *__restrict__ stb, const typename V4<
 #pragma unroll
         for (int t2 = 0; t2 < 5; ++t2) {
             const T y[4] = {st.th[1][t2], st.d1[1][t2], st.d2[1][t2], st.d3[1][t2]};
-            const T *row = phi + ((size_t)st.k[2][t3] * Ky + st.k[1][t2]) * Kx;
-            T S[4] = {0, 0, 0, 0};
-#pragma unroll
-            for (int t1 = 0; t1 < 5; ++t1) {
-                const T v = row[st.k[0][t1]];
-                S[0] += st.th[0][t1] * v;
-                S[1] += st.d1[0][t1] * v;
-                S[2] += st.d2[0][t1] * v;
-                S[3] += st.d3[0][t1] * v;
-            }
+            T S[4];
+            rx.sums(phi + ((size_t)st.k[2][t3] * Ky + st.k[1][t2]) * Kx, S);
             D[0] += S[0] * y[0] * z[0];
             D[1] += S[1] * y[0] * z[0];
             D[2] += S[0] * y[1] * z[0];
@@ -543,7 +628,16 @@ int gather_launch(ap_ctx *ctx, const T *phi, T *out, cudaStream_t s) {
     typedef typename V4<T>::type T4;
     PmeConsts<T> pc = pme_consts<T>(ctx);
     const int th = ctx->tune_pme_threads;
-    k_gather_field<T><<<ap_grid_for(ctx->n, th), th, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, phi, out, ctx->n_pad, pc);
+    const bool wide = sizeof(T) == 4 && ctx->K[0] % 4 == 0;
+    // five threads per atom while they make at most one wave of the GPU's thread slots (wide, one -> five: 9.8
+    // -> 6.1 us at 648 atoms, 10.0 -> 7.9 at 12,288, 11.9 -> 11.1 at 22,969; 14.2 -> 21.2 at 96,000)
+    if (5L * ctx->n <= 2048L * ctx->sm_count) {
+        auto kern = wide ? k_gather_field5<T, true> : k_gather_field5<T, false>;
+        kern<<<lane5_blocks(ctx->n, th), th, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, phi, out, ctx->n_pad, pc);
+    } else {
+        auto kern = wide ? k_gather_field<T, true> : k_gather_field<T, false>;
+        kern<<<ap_grid_for(ctx->n, th), th, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, phi, out, ctx->n_pad, pc);
+    }
     AP_CUDA(cudaGetLastError());
     return AP_OK;
 }
@@ -757,10 +851,12 @@ int forces_t(ap_ctx *ctx, const void *mu4, double *gbuf, int with_M, cudaStream_
             else AP_CUFFT(cufftExecC2R(bf.c2r, (cufftComplex *)ctx->cgrid, (cufftReal *)ctx->grid));
         }
     }
-    k_gather_derivs<T><<<ap_grid_for(ctx->n, 128), 128, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, (const T *)ctx->grid,
+    const bool wide = sizeof(T) == 4 && ctx->K[0] % 4 == 0;
+    auto derivs = wide ? k_gather_derivs<T, true> : k_gather_derivs<T, false>;
+    derivs<<<ap_grid_for(ctx->n, 128), 128, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, (const T *)ctx->grid,
                                                                gbuf, ctx->n_pad, 20, pc);
     if (with_M)
-        k_gather_derivs<T><<<ap_grid_for(ctx->n, 128), 128, 0, s>>>(ctx->stb, (const T4 *)ctx->stw,
+        derivs<<<ap_grid_for(ctx->n, 128), 128, 0, s>>>(ctx->stb, (const T4 *)ctx->stw,
                                                                    (const T *)ctx->grid2,
                                                                    gbuf + (size_t)20 * ctx->n_pad, ctx->n_pad, 10, pc);
     else
