@@ -474,6 +474,163 @@ __global__ void k_spread_multipoles5(const typename V4<T>::type *__restrict__ po
     }
 }
 
+// Large systems: the FP32 dipole spread through a box in shared memory. A warp takes a block of 32
+// atoms; its box is the grid region of their stencils. Atom after atom, lane t2 + 5 t3 adds that row's
+// five points to the box (plain loads and stores: a row belongs to one lane, and the pitches put the
+// 25 rows on 25 banks), four atoms' rows formed ahead of them; then the box goes to the grid with
+// four-wide reductions. The kernels above send every atom's 25 rows to the L2 as two or three reductions
+// each, and its reduction rate bounds them; here 32 atoms of water at a grid spacing of 1 A share about 650
+// reductions instead of 1,800. Bound by the latency of a warp's adds (about 10 warps per SM).
+// Measured on GB300: 38.2 -> 27.4 us at 96,000 atoms (an iteration of the solve 108.1 -> 97.4),
+// 277 -> 182 us at 1,065,000 (1069 -> 992). The carveout matters: the kernel runs beside the pair kernel, and with
+// the driver's choice (all of it for shared memory) that keeps off its SMs: 1,065,000 atoms 1016 us, with two
+// blocks a warp 1219.
+constexpr int BOX_FLOATS = 3584, BOX_CARVEOUT = 80;
+constexpr int BOX_PITCH = 36;   // floats per atom record; 4 mod 8: conflict-free 16-byte stores
+
+__global__ void __launch_bounds__(32) k_spread_box(const float4 *__restrict__ dip, const int4 *__restrict__ stb,
+                                                   const float4 *__restrict__ stw, float *__restrict__ grid,
+                                                   PmeConsts<float> pc) {
+    __shared__ __align__(16) float rec[32 * BOX_PITCH];
+    __shared__ __align__(16) float box[BOX_FLOATS];
+    const int lane = threadIdx.x;
+    const unsigned full = 0xffffffffu;
+    const int first = blockIdx.x * 32, m = min(32, pc.n - first);
+    const int Kx = pc.K[0], Ky = pc.K[1], Kz = pc.K[2];
+    const int i = first + min(lane, m - 1);
+    const int4 b = stb[i], ref = stb[first];
+    const float4 w = stw[i], u = dip[i];
+    // origin relative to the first atom's, nearest image
+    auto rel = [](int b, int r, int K) {
+        int v = b - r;
+        if (2 * v >= K) v -= K;
+        if (2 * v < -K) v += K;
+        return v;
+    };
+    const int org[3] = {rel(b.x, ref.x, Kx), rel(b.y, ref.y, Ky), rel(b.z, ref.z, Kz)};
+    // first point of the box (relative to the first atom's origin; along x on a multiple of four of the
+    // grid, Kx being one), points, pitches of rows and planes
+    int lo[3], hi[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        lo[d] = __reduce_min_sync(full, org[d]) - 4;
+        hi[d] = __reduce_max_sync(full, org[d]);
+    }
+    lo[0] -= (ref.x + lo[0] + 2 * Kx) & 3;
+    const int W = (hi[0] - lo[0] + 4) & ~3, H = hi[1] - lo[1] + 1, D = hi[2] - lo[2] + 1;
+    // row (t2, t3) of a stencil R (t2 + 5 t3) banks on: R odd, P = 5 R modulo 32
+    const int R = W | 1, P = H * R + (((5 - H) * R) & 31);
+    const bool boxed = (long long)P * D <= BOX_FLOATS;   // else (atoms strewn over the grid) row by row to the grid
+    if (boxed)
+        for (int q = 4 * lane; q < P * D; q += 128) *reinterpret_cast<float4 *>(box + q) = make_float4(0.f, 0.f, 0.f, 0.f);
+    {
+        // the atom's record: weight and derivative times dipole of each of the five points per
+        // dimension, its place in the box
+        float th[3][5], d1[3][5], *none = nullptr;
+        bspline5<float, 1>(w.x, th[0], d1[0], none, none);
+        bspline5<float, 1>(w.y, th[1], d1[1], none, none);
+        bspline5<float, 1>(w.z, th[2], d1[2], none, none);
+        const float mu[3] = {u.x * pc.s[0], u.y * pc.s[1], u.z * pc.s[2]};
+        float r[32];
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+#pragma unroll
+            for (int t = 0; t < 5; ++t) {
+                r[(d * 5 + t) * 2] = th[d][t];
+                r[(d * 5 + t) * 2 + 1] = mu[d] * d1[d][t];
+            }
+        r[30] = __int_as_float((org[2] - lo[2]) * P + (org[1] - lo[1]) * R + org[0] - lo[0]);
+        r[31] = 0.f;
+#pragma unroll
+        for (int q = 0; q < 32; q += 4)
+            *reinterpret_cast<float4 *>(rec + lane * BOX_PITCH + q) = make_float4(r[q], r[q + 1], r[q + 2], r[q + 3]);
+    }
+    __syncwarp();
+    // the five points of row (t2, t3) of an atom
+    const int t3 = min(lane / 5, 4), t2 = lane - 5 * (lane / 5);
+    const bool row = lane < 25;
+    auto values = [&](const float *q, float *v) {
+        const float2 y = *reinterpret_cast<const float2 *>(q + 10 + 2 * t2), z = *reinterpret_cast<const float2 *>(q + 20 + 2 * t3);
+        const float4 xa = *reinterpret_cast<const float4 *>(q), xb = *reinterpret_cast<const float4 *>(q + 4);
+        const float2 xc = *reinterpret_cast<const float2 *>(q + 8);
+        const float A = y.y * z.x + y.x * z.y, C = y.x * z.x;
+        v[0] = xa.x * A + xa.y * C;
+        v[1] = xa.z * A + xa.w * C;
+        v[2] = xb.x * A + xb.y * C;
+        v[3] = xb.z * A + xb.w * C;
+        v[4] = xc.x * A + xc.y * C;
+    };
+    if (!boxed) {
+        for (int a = 0; a < m; ++a) {
+            const int4 o = stb[first + a];
+            float v[5];
+            values(rec + a * BOX_PITCH, v);
+            if (row) {
+                const int ky = o.y - t2, kz = o.z - t3;
+                int k[5];
+#pragma unroll
+                for (int t = 0; t < 5; ++t) k[t] = o.x - t < 0 ? o.x - t + Kx : o.x - t;
+                add_row5(grid + ((size_t)(kz < 0 ? kz + Kz : kz) * Ky + (ky < 0 ? ky + Ky : ky)) * Kx, k, v, Kx);
+            }
+        }
+        return;
+    }
+    const int mine = t3 * P + t2 * R;
+    constexpr int U = 4;   // rows formed ahead of the box's loads and stores
+    for (int a = 0; a < m; a += U) {
+        float v[U][5];
+        float *at[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            const float *q = rec + min(a + j, m - 1) * BOX_PITCH;
+            at[j] = box + (row ? __float_as_int(q[30]) - mine : 4);
+            values(q, v[j]);
+        }
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            if (row && a + j < m) {
+                float o[5];
+#pragma unroll
+                for (int t = 0; t < 5; ++t) o[t] = at[j][-t];
+#pragma unroll
+                for (int t = 0; t < 5; ++t) at[j][-t] = o[t] + v[j][t];
+            }
+            __syncwarp();
+        }
+    }
+    const int cols = W / 4, items = cols * H * D;
+    const float icols = 1.f / cols, iH = 1.f / H;   // quotients of integers below 2^12: exact with the half
+    int o[3] = {(ref.x + lo[0]) % Kx, (ref.y + lo[1]) % Ky, (ref.z + lo[2]) % Kz};
+    o[0] += o[0] < 0 ? Kx : 0;
+    o[1] += o[1] < 0 ? Ky : 0;
+    o[2] += o[2] < 0 ? Kz : 0;
+#pragma unroll 4
+    for (int q = lane; q < items; q += 32) {
+        const int yz = (int)((q + 0.5f) * icols), c = 4 * (q - yz * cols);
+        const int z = (int)((yz + 0.5f) * iH), y = yz - z * H;
+        int gx = o[0] + c, gy = o[1] + y, gz = o[2] + z;
+        while (gx >= Kx) gx -= Kx;
+        while (gy >= Ky) gy -= Ky;
+        while (gz >= Kz) gz -= Kz;
+        const float *f = box + z * P + y * R + c;
+        atomicAdd(reinterpret_cast<float4 *>(grid + ((size_t)gz * Ky + gy) * Kx + gx), make_float4(f[0], f[1], f[2], f[3]));
+    }
+}
+
+// Whether the dipole spread goes through boxes: floating-point sums, rows of a multiple of four points, at
+// least BOX_MIN blocks per SM (a warp's chain of adds takes 15 us, which few blocks do not fill; direct -> boxes
+// 11.3 -> 15.4 us at 95 blocks, an iteration 61.5 -> 64.2 at 461, 47.6 -> 48.9 at 547, 54.4 -> 50.9 at 644, 58.8 -> 53.7
+// at 750), and a grid so coarse that a block of evenly spread atoms, a cube of 32 atoms a quarter longer
+// along x, has its box in BOX_FLOATS (one that does not fit spreads with a warp's 25 lanes an atom, slower
+// than the kernels above).
+constexpr double BOX_MIN = 4.0;
+bool spread_boxed(const ap_ctx *ctx) {
+    if (ctx->prec == AP_FP64 || ctx->fixed || ctx->K[0] % 4 || ctx->n_blocks < BOX_MIN * ctx->sm_count) return false;
+    const double *L = ctx->prm.box, side = std::cbrt(32.0 * L[0] * L[1] * L[2] / ctx->n);
+    const double x = 1.25 * side * ctx->K[0] / L[0] + 7.5, y = side * ctx->K[1] / L[1] + 5.5, z = side * ctx->K[2] / L[2] + 5.5;
+    return 1.1 * x * y * z <= BOX_FLOATS;
+}
+
 // derivatives of phi up to third order (20 components) for the forces -------------------
 // component order: [0] phi; [1..3] x y z; [4..9] xx yy zz xy xz yz;
 // [10..19] xxx yyy zzz xxy xxz xyy yyz xzz yzz xyz
@@ -590,6 +747,7 @@ int init_t(ap_ctx *ctx) {
     AP_CUDA(cudaMemcpy(ctx->green, g.data(), sizeof(T) * g.size(), cudaMemcpyHostToDevice));
     bool dbl = sizeof(T) == 8;
     if constexpr (std::is_same<T, float>::value) {
+        AP_CUDA(cudaFuncSetAttribute(k_spread_box, cudaFuncAttributePreferredSharedMemoryCarveout, BOX_CARVEOUT));
         if (fft_supported(ctx)) {
             const int r = fft_init(ctx, g.data());
             if (r) return r;
@@ -677,6 +835,13 @@ int spread_t(ap_ctx *ctx, const PmeBufs &bf, const void *src, bool multi, cudaSt
     // five threads per atom while they make at most two waves of the GPU's thread slots
     const bool five = 5L * ctx->n <= 2L * 2048 * ctx->sm_count;
     if (!fx && !cleared) AP_CUDA(cudaMemsetAsync(bf.grid, 0, sizeof(T) * ctx->ngrid, s));
+    if constexpr (std::is_same<T, float>::value) {
+        if (!multi && spread_boxed(ctx)) {
+            k_spread_box<<<ctx->n_blocks, 32, 0, s>>>((const float4 *)src, ctx->stb, (const float4 *)ctx->stw, (float *)g, pc);
+            AP_CUDA(cudaGetLastError());
+            return AP_OK;
+        }
+    }
     if (multi) {
         if (five) {
             auto kern = fx ? k_spread_multipoles5<T, true> : k_spread_multipoles5<T, false>;
