@@ -287,8 +287,8 @@ def pairs_within(xyz, box, rc):
 def launches_per_step(iters, n, rebuild_frac, guess_launches):
     """Kernels of this library launched by one step (cuFFT's own kernels not counted)."""
     pad = 1 if n % 32 else 0
-    field = 8 + pad + 5                   # load, filter, work offsets, work fill, pair masks, 3 prefix
-    #                                       scans, [pad]; spread, convolve, gather, pair field, assemble
+    field = 7 + pad                       # load, pair lists, [pad]; spread, convolve, gather, pair field,
+    #                                       assemble
     guess = guess_launches
     solve = 1 + 4 + 1 + 1 + 7 * iters + 1  # guess, matvec(4), residual (+ state), cond, 7/iter, unsort
     forces = 10
