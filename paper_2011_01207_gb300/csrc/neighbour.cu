@@ -190,56 +190,91 @@ __global__ void k_block_bbox(const double *__restrict__ xyz, const int *__restri
     }
 }
 
-__device__ __forceinline__ bool blocks_near(float4 ci, float4 hi, float4 cj, float4 hj, float3 L, float r2) {
-    float dx = ci.x - cj.x, dy = ci.y - cj.y, dz = ci.z - cj.z;
-    dx -= L.x * rintf(dx / L.x);
-    dy -= L.y * rintf(dy / L.y);
-    dz -= L.z * rintf(dz / L.z);
-    float gx = fmaxf(0.f, fabsf(dx) - hi.x - hj.x);
-    float gy = fmaxf(0.f, fabsf(dy) - hi.y - hj.y);
-    float gz = fmaxf(0.f, fabsf(dz) - hi.z - hj.z);
+// centres lie in [0, L), so min(|d|, L - |d|) is the nearest image's distance
+__device__ __forceinline__ bool blocks_near(const float4 &ci, const float4 &hi, const float4 &cj, const float4 &hj, const float3 &L,
+                                            float r2) {
+    const float ax = fabsf(ci.x - cj.x), ay = fabsf(ci.y - cj.y), az = fabsf(ci.z - cj.z);
+    const float gx = fmaxf(0.f, fminf(ax, L.x - ax) - hi.x - hj.x);
+    const float gy = fmaxf(0.f, fminf(ay, L.y - ay) - hi.y - hj.y);
+    const float gz = fmaxf(0.f, fminf(az, L.z - az) - hi.z - hj.z);
     return gx * gx + gy * gy + gz * gz < r2;
 }
 
-// one warp per block I: count (tiles == nullptr) or write its partners J, I among them (as many as
-// fit: the caller looks at the total and grows the arrays)
+// One warp per TILE_I blocks I: count (tiles == nullptr) or write their partners J, I among them (as
+// many as fit: the caller looks at the total and grows the arrays). Two blocks per warp halve the
+// loads of J, and four of those are in flight per lane. (With one block a warp, a division per dimension and the
+// tiles' FP64 origins formed here by the few lanes that hit, a build and field took 625 us for 554 at 96,000 atoms
+// and 4,064 for 3,605 at 648,000.)
+constexpr int TILE_I = 2;
 __global__ void k_tiles(const float4 *__restrict__ center, const float4 *__restrict__ half, int nb,
                         float3 L, float r2, int *__restrict__ count, const int *__restrict__ off,
-                        TileRec *__restrict__ tiles, int cap, double3 Ld) {
-    int I = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (I >= nb) return;
-    float4 ci = center[I], hi = half[I];
-    int pos = tiles ? off[I] : 0;
-    int cnt = 0;
-    for (int base = 0; base < nb; base += 32) {
-        int J = base + lane;
-        bool hit = false;
-        if (J < nb) hit = blocks_near(ci, hi, center[J], half[J], L, r2);
-        unsigned m = __ballot_sync(0xffffffffu, hit);
-        const int k = pos + __popc(m & ((1u << lane) - 1u));
-        if (tiles && hit && k < cap) {
-            const float4 cj = center[J];
-            // origin of J's image next to I, relative to I's origin: c_J - c_I + L k in FP64,
-            // split into float hi + lo (the centres are the blocks' position origins)
-            const double ox = (double)cj.x - (double)ci.x + Ld.x * rintf((ci.x - cj.x) / L.x);
-            const double oy = (double)cj.y - (double)ci.y + Ld.y * rintf((ci.y - cj.y) / L.y);
-            const double oz = (double)cj.z - (double)ci.z + Ld.z * rintf((ci.z - cj.z) / L.z);
-            TileRec r;
-            r.J = J;
-            r.excl = -1;
-            r.hx = (float)ox;
-            r.hy = (float)oy;
-            r.hz = (float)oz;
-            r.lx = (float)(ox - r.hx);
-            r.ly = (float)(oy - r.hy);
-            r.lz = (float)(oz - r.hz);
-            tiles[k] = r;
-        }
-        pos += __popc(m);
-        cnt += __popc(m);
+                        TileRec *__restrict__ tiles, int cap) {
+    const int I0 = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) * TILE_I;
+    const int lane = threadIdx.x & 31;
+    if (I0 >= nb) return;
+    float4 ci[TILE_I], hi[TILE_I];
+    int pos[TILE_I];
+#pragma unroll
+    for (int i = 0; i < TILE_I; ++i) {
+        const int I = min(I0 + i, nb - 1);
+        ci[i] = center[I];
+        hi[i] = half[I];
+        pos[i] = tiles ? off[I] : 0;
     }
-    if (!tiles && lane == 0) count[I] = cnt;
+    constexpr int U = 4;
+    for (int base = 0; base < nb; base += 32 * U) {
+        float4 cj[U], hj[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int J = min(base + 32 * u + lane, nb - 1);
+            cj[u] = center[J];
+            hj[u] = half[J];
+        }
+#pragma unroll
+        for (int i = 0; i < TILE_I; ++i) {
+            if (I0 + i >= nb) break;
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int J = base + 32 * u + lane;
+                const bool hit = blocks_near(ci[i], hi[i], cj[u], hj[u], L, r2) && J < nb;
+                const unsigned m = __ballot_sync(0xffffffffu, hit);
+                const int k = pos[i] + __popc(m & ((1u << lane) - 1u));
+                if (tiles && hit && k < cap) {
+                    TileRec r = {};
+                    r.J = J;
+                    r.excl = I0 + i;   // until k_tile_origins
+                    tiles[k] = r;
+                }
+                pos[i] += __popc(m);
+            }
+        }
+    }
+    if (!tiles && lane == 0)
+#pragma unroll
+        for (int i = 0; i < TILE_I; ++i)
+            if (I0 + i < nb) count[I0 + i] = pos[i];
+}
+
+// The tiles' origins, one thread each: J's image next to I relative to I's origin, c_J - c_I + L k in
+// FP64, split into float hi + lo (the centres are the blocks' position origins). Apart from k_tiles, where
+// a few lanes of a warp at a time ran these FP64 instructions.
+__global__ void k_tile_origins(const float4 *__restrict__ center, float3 L, double3 Ld, const int *__restrict__ total, int cap,
+                               TileRec *__restrict__ tiles) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= min(*total, cap)) return;
+    TileRec r = tiles[t];
+    const float4 a = center[r.excl], c = center[r.J];
+    const double ox = (double)c.x - (double)a.x + Ld.x * rintf((a.x - c.x) / L.x);
+    const double oy = (double)c.y - (double)a.y + Ld.y * rintf((a.y - c.y) / L.y);
+    const double oz = (double)c.z - (double)a.z + Ld.z * rintf((a.z - c.z) / L.z);
+    r.excl = -1;
+    r.hx = (float)ox;
+    r.hy = (float)oy;
+    r.hz = (float)oz;
+    r.lx = (float)(ox - r.hx);
+    r.ly = (float)(oy - r.hy);
+    r.lz = (float)(oz - r.hz);
+    tiles[t] = r;
 }
 
 __device__ int find_tile(const TileRec *__restrict__ tiles, int b, int e, int J) {
@@ -350,8 +385,8 @@ int nb_build(ap_ctx *ctx, const double *d_xyz, const int *d_off, const int *d_at
     const float3 L = make_float3((float)P.box[0], (float)P.box[1], (float)P.box[2]);
     const float rl = (float)(P.cutoff + P.buffer);
     int *bcount = key;                 // reuse: key no longer needed
-    const int warps = ap_grid_for((long)nb * 32, T);
-    k_tiles<<<warps, T, 0, s>>>(ctx->bcenter, ctx->bhalf, nb, L, rl * rl, bcount, nullptr, nullptr, 0, Ld);
+    const int warps = ap_grid_for((long)(nb + TILE_I - 1) / TILE_I * 32, T);
+    k_tiles<<<warps, T, 0, s>>>(ctx->bcenter, ctx->bhalf, nb, L, rl * rl, bcount, nullptr, nullptr, 0);
     k_scan_single<<<1, 1024, 0, s>>>(bcount, ctx->tile_off, nb, info + NB_TILES);
     AP_CUDA(cudaGetLastError());
 
@@ -363,7 +398,9 @@ int nb_build(ap_ctx *ctx, const double *d_xyz, const int *d_off, const int *d_at
     for (int round = 0;; ++round) {
         if (ctx->cap_tiles > 0) {
             k_tiles<<<warps, T, 0, s>>>(ctx->bcenter, ctx->bhalf, nb, L, rl * rl, nullptr, ctx->tile_off, ctx->tiles,
-                                        ctx->cap_tiles, Ld);
+                                        ctx->cap_tiles);
+            k_tile_origins<<<ap_grid_for(ctx->cap_tiles, T), T, 0, s>>>(ctx->bcenter, L, Ld, info + NB_TILES, ctx->cap_tiles,
+                                                                       ctx->tiles);
             if (n_excl > 0) {
                 const int slots = ctx->cap_excl / 32;
                 AP_CUDA(cudaMemsetAsync(info + NB_FAR, 0, sizeof(int) * 3, s));
