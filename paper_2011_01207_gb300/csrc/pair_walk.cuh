@@ -113,15 +113,20 @@ struct Layout {
     }
 };
 
-// the targets of a thread, and the limits of their r^2 (negative for padding)
+// The targets of a thread, and the limits of their r^2 (negative for padding). In FP32 a padding slot can be
+// the other half of a real atom's pair, and its terms are evaluated with the rest: it lies far from every
+// candidate and from the phantom, so that r^2 is neither zero nor beyond FP32 and the zero exponentials of a pair
+// out of range make each of its terms exactly zero. (At the block's origin, where the middle atom of a
+// molecule can lie, 1/r is infinite and the slot's sums NaN.)
+constexpr float PADDING_AT = 1e6f;
 template <class T> struct Targets;
 template <> struct Targets<float> {
     float2 x, y, z, w, lim;
     __device__ __forceinline__ void load(const float4 *posw, int s0, int, int n, float rc2, float ta) {
         float4 a = posw[s0], b = posw[s0 + 1];
         const bool va = s0 < n, vb = s0 + 1 < n;
-        if (!va) a.x = a.y = a.z = 0.f;
-        if (!vb) b.x = b.y = b.z = 0.f;
+        if (!va) a.x = a.y = a.z = PADDING_AT;
+        if (!vb) b.x = b.y = b.z = PADDING_AT;
         x = make_float2(a.x, b.x);
         y = make_float2(a.y, b.y);
         z = make_float2(a.z, b.z);
