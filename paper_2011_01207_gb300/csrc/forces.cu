@@ -9,7 +9,8 @@
 //               potentials' derivatives up to third order at the atoms;
 //   frames:     global multipoles rotate with their frame atoms: dU/d(global dipole) and
 //               dU/d(global quadrupole) are chained through the frame construction.
-// Pair arithmetic in T, accumulation in FP64 as in the other real-space kernels.
+// Pair arithmetic in T; a thread's sums over its pairs in T; those over a target's threads, and what its own
+// multipoles make of them, in FP64 or compensated FP32 pairs.
 //
 // Virial (on request): V_ab = dE_pol/de_ab under x -> (I + e) x of positions and box, which
 // the paper's real-space loop updates with the energy and the forces (Sec. 1.2.1) and sums in
@@ -86,6 +87,8 @@ __device__ __forceinline__ void block_add9(V *v, double *acc) {
 // Measured on GB300 (ncu, warm): 228 -> 134.7 us at 96,000 atoms, 44.2 -> 23.5 us at 6,000, against
 // contracting both atoms' multipoles per pair side on 32 x 32 pair masks. 159 registers, so 3 CTAs
 // per SM (shared memory would hold 4): what bounds it is issue at that occupancy.
+// (Timed with events, of the 136.1 us at 96,000 atoms the compensated sums of a target's threads take 2.5 and the
+// compensated contraction 1.5.)
 // Every term is linear in the R_n, which come negated, so the sums are those of -E and -G.
 // Excluded pairs (sigma = 0 between permanent and induced, 1 between induced and induced) come
 // first in the lists and take two sets of radial functions.
@@ -96,7 +99,20 @@ struct FieldSums {
     V gxx, gyy, gzz, gxy, gxz, gyz, gtr;             // G: the diagonal's t_a R_a part halved
     V qxx, qyy, qzz;                                 // and the diagonal of -(2/3) R2 Q
 };
-constexpr int FS = 33;
+constexpr int FS = 33, FO = 29;
+// what the force is made of: E, E_ab (the diagonal halved, without its trace part) and that part, S, W, and G whole
+template <class Vt>
+__device__ __forceinline__ void fold(const FieldSums<Vt> &a, Vt *o) {
+    const Vt *v = reinterpret_cast<const Vt *>(&a);
+#pragma unroll
+    for (int k = 0; k < 23; ++k) o[k] = v[k];
+    o[23] = add2(add2(a.gxx, a.gxx), add2(a.gtr, a.qxx));
+    o[24] = add2(add2(a.gyy, a.gyy), add2(a.gtr, a.qyy));
+    o[25] = add2(add2(a.gzz, a.gzz), add2(a.gtr, a.qzz));
+    o[26] = a.gxy;
+    o[27] = a.gxz;
+    o[28] = a.gyz;
+}
 
 template <class T>
 __device__ __forceinline__ void zero_sums(FieldSums<typename Vec<T>::type> &a) {
@@ -192,13 +208,12 @@ template <class X>
 struct OwnPoles {
     X q, d[3], Q[6], mu[3];
 };
-// force (over f) of those multipoles in the fields of the sums a[0..FS-1] (order of FieldSums)
-template <class X>
-__device__ __forceinline__ void own_force(const X *a, const OwnPoles<X> &m, X *F) {
-    const X tr = a[9], g = a[29];
+// component C of the force (over f) of those multipoles in the fields of the sums a[0..FO-1] (order of fold)
+template <int C, class X>
+__device__ __forceinline__ X own_force(const X *a, const OwnPoles<X> &m) {
+    const X tr = a[9];
     const X Eab[3][3] = {{2 * a[3] + tr, a[6], a[7]}, {a[6], 2 * a[4] + tr, a[8]}, {a[7], a[8], 2 * a[5] + tr}};
-    const X G[3][3] = {{2 * a[23] + a[30] + g, a[26], a[27]}, {a[26], 2 * a[24] + a[31] + g, a[28]},
-                       {a[27], a[28], 2 * a[25] + a[32] + g}};
+    const X G[3][3] = {{a[23], a[26], a[27]}, {a[26], a[24], a[28]}, {a[27], a[28], a[25]}};
     const X *S = a + 10, *W = a + 20, *Q = m.Q;
     // sum_bc Q_bc E_abc, with sum_bc Q_bc delta_bc = 0
     const X QS[3] = {Q[0] * 3 * S[0] + Q[3] * S[5] + Q[5] * S[7] + 2 * (Q[1] * S[3] + Q[2] * S[4] + Q[4] * S[9]),
@@ -206,10 +221,42 @@ __device__ __forceinline__ void own_force(const X *a, const OwnPoles<X> &m, X *F
                      Q[0] * S[4] + Q[3] * S[6] + Q[5] * 3 * S[2] + 2 * (Q[1] * S[9] + Q[2] * S[7] + Q[4] * S[8])};
     const X QW[3] = {Q[0] * W[0] + Q[1] * W[1] + Q[2] * W[2], Q[1] * W[0] + Q[3] * W[1] + Q[4] * W[2],
                      Q[2] * W[0] + Q[4] * W[1] + Q[5] * W[2]};
+    return m.q * a[C] + m.d[0] * Eab[0][C] + m.d[1] * Eab[1][C] + m.d[2] * Eab[2][C] + (QS[C] + 2 * QW[C]) * X(1.0 / 3.0) +
+           m.mu[0] * G[0][C] + m.mu[1] * G[1][C] + m.mu[2] * G[2][C];
+}
+
+// The same from sums in compensated FP32 pairs (hi, lo): every product with hi exact (its rounding error by an
+// fma) and added to a compensated pair, the quadrupole's terms apart for their factor of a third.
+struct WideDot {
+    F2 s = {0.f, 0.f};
+    __device__ __forceinline__ void add(float c, float2 a) {
+        const float p = c * a.x;
+        f2_add(s, p);
+        s.lo += fmaf(c, a.y, fmaf(c, a.x, -p));
+    }
+    __device__ __forceinline__ double value() const { return f2d_exact(s.hi) + f2d_exact(s.lo); }
+};
+template <int C>
+__device__ __forceinline__ double own_force_wide(const float2 *a, const OwnPoles<float> &m) {
+    constexpr int X = (C + 1) % 3, Y = (C + 2) % 3;             // the other two components
+    constexpr int AT[3][3] = {{0, 6, 7}, {6, 0, 8}, {7, 8, 0}};   // xy, xz, yz in E_ab; 20 further in G
+    constexpr int S3[3][6] = {{0, 5, 7, 3, 4, 9}, {3, 1, 8, 5, 9, 6}, {4, 6, 2, 9, 7, 8}};   // of Q xx yy zz xy xz yz
+    constexpr int QI[6] = {0, 3, 5, 1, 2, 4}, QR[3][3] = {{0, 1, 2}, {1, 3, 4}, {2, 4, 5}};
+    WideDot f, t;
+    f.add(m.q, a[C]);
+    f.add(2 * m.d[C], a[3 + C]);
+    f.add(m.d[C], a[9]);
+    f.add(m.d[X], a[AT[C][X]]);
+    f.add(m.d[Y], a[AT[C][Y]]);
+    f.add(m.mu[C], a[23 + C]);
+    f.add(m.mu[X], a[20 + AT[C][X]]);
+    f.add(m.mu[Y], a[20 + AT[C][Y]]);
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-        F[c] = m.q * a[c] + m.d[0] * Eab[0][c] + m.d[1] * Eab[1][c] + m.d[2] * Eab[2][c] +
-               (QS[c] + 2 * QW[c]) * X(1.0 / 3.0) + m.mu[0] * G[0][c] + m.mu[1] * G[1][c] + m.mu[2] * G[2][c];
+    for (int k = 0; k < 6; ++k) t.add((k < 3 ? 1 : 2) * m.Q[QI[k]], a[10 + S3[C][k]]);
+    t.add(2 * m.Q[QI[C]], a[10 + C]);   // the diagonal's are kept as a third
+#pragma unroll
+    for (int k = 0; k < 3; ++k) t.add(2 * m.Q[QR[C][k]], a[20 + k]);
+    return f.value() + t.value() * (1.0 / 3.0);
 }
 
 template <class T>
@@ -258,15 +305,20 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !VIR ? 3 : 1) k_pair_for
     FieldSums<Vt> sum;
     zero_sums<T>(sum);
     OwnPoles<T> own[W];
-    Vt vs[9];                       // sum of F R^T over this thread's sides (VIR)
+    Vt vs[9];                       // sum of F R^T over this thread's sides of a chunk (VIR)
+    double vsum[9];                 // and over all chunks
     if constexpr (VIR) {
 #pragma unroll
         for (int h = 0; h < W; ++h) own[h] = own_poles<T>(src, ly.slot() + h, pc.n);
 #pragma unroll
-        for (int k = 0; k < 9; ++k) vs[k] = splat2(T(0));
+        for (int k = 0; k < 9; ++k) vsum[k] = 0.0;
     }
     const T4 *const from[4] = {src.dipd, src.quad0, src.quad1, src.mu};
     for_chunks<T, PARTS>(raw, la, ly, from, [&](const unsigned *list, int words, int flagged, int) {
+        if constexpr (VIR) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) vs[k] = splat2(T(0));
+        }
         auto side = [&](unsigned e, auto ex) {
             constexpr bool EX = decltype(ex)::value;
             const unsigned char *at = raw + (e & 0xfff0u) * (unsigned)(sizeof(T4) / 16);
@@ -293,18 +345,22 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !VIR ? 3 : 1) k_pair_for
                 FieldSums<Vt> one;
                 zero_sums<T>(one);
                 add(one);
-                const Vt *o1 = reinterpret_cast<const Vt *>(&one);
                 if constexpr (W == 1) {
+                    const Vt *o1 = reinterpret_cast<const Vt *>(&one);
                     Vt *t = reinterpret_cast<Vt *>(&sum);
 #pragma unroll
                     for (int k = 0; k < FS; ++k) t[k] = add2(t[k], o1[k]);
                 }
+                Vt of[FO];
+                fold(one, of);
 #pragma unroll
                 for (int h = 0; h < W; ++h) {
-                    T v[FS], F[3];
+                    T v[FO], F[3];
 #pragma unroll
-                    for (int k = 0; k < FS; ++k) v[k] = Vec<T>::get(o1[k], h);
-                    own_force<T>(v, own[h], F);
+                    for (int k = 0; k < FO; ++k) v[k] = Vec<T>::get(of[k], h);
+                    F[0] = own_force<0>(v, own[h]);
+                    F[1] = own_force<1>(v, own[h]);
+                    F[2] = own_force<2>(v, own[h]);
 #pragma unroll
                     for (int x = 0; x < 3; ++x)
 #pragma unroll
@@ -317,51 +373,86 @@ __global__ void __launch_bounds__(FT, sizeof(T) == 4 && !VIR ? 3 : 1) k_pair_for
         };
         walk(list, words, flagged, ly.first, ly.STRIDE, [&](unsigned e) { side(e, std::true_type()); },
              [&](unsigned e) { side(e, std::false_type()); });
-    });
-    // the sums of a target's threads through shared memory (the staged candidates are done with):
-    // number k of target h at red[(W k + h) FT + tid]
-    __syncthreads();
-    T *red = reinterpret_cast<T *>(raw), *tot = red + W * FS * FT;
-    {
-        const Vt *v = reinterpret_cast<const Vt *>(&sum);
+        if constexpr (VIR) {
 #pragma unroll
-        for (int k = 0; k < FS; ++k)
+            for (int k = 0; k < 9; ++k) {
+                vsum[k] += (double)Vec<T>::get(vs[k], 0);
+                if (W == 2) vsum[k] += (double)Vec<T>::get(vs[k], 1);
+            }
+        }
+    });
+    // The sums of a target's threads through shared memory (the staged candidates are done with): number k
+    // of target h at red[(W k + h) FT + tid]. In FP32 they are compensated pairs, and so is what the target's own
+    // multipoles make of them.
+    __syncthreads();
+    T *red = reinterpret_cast<T *>(raw);
+    Vt *tot = reinterpret_cast<Vt *>(red + W * FO * FT);
+    {
+        Vt v[FO];
+        fold(sum, v);
+#pragma unroll
+        for (int k = 0; k < FO; ++k)
 #pragma unroll
             for (int h = 0; h < W; ++h) red[(W * k + h) * FT + threadIdx.x] = Vec<T>::get(v[k], h);
     }
     __syncthreads();
     constexpr int NT = 2 * LY::PAIRS;   // targets of this CTA
-    for (int q = threadIdx.x; q < FS * NT; q += FT) {
-        const int k = q / NT, t = q % NT, pp = t >> 1, h = t & 1;
-        const T *r = red + (W == 2 ? 2 * k + h : k) * FT + pp * LY::TP + (W == 2 ? 0 : h);
-        T v = T(0);
+    if constexpr (W == 2) {
+        for (int q = threadIdx.x; q < FO * LY::PAIRS; q += FT) {
+            const int k = q / LY::PAIRS, pp = q % LY::PAIRS;
+            const float *r = red + 2 * k * FT + pp * LY::TP;
+            float2 hi = make_float2(0.f, 0.f), lo = hi;
 #pragma unroll
-        for (int i = 0; i < LY::TP; i += W == 2 ? 1 : 2) v += r[i];
-        tot[t * (FS + 1) + k] = v;
+            for (int i = 0; i < LY::TP; i += 4) {
+                const float4 a = *reinterpret_cast<const float4 *>(r + i), b = *reinterpret_cast<const float4 *>(r + FT + i);
+                if (i) f2_add(hi, lo, make_float2(a.x, b.x));
+                else hi = make_float2(a.x, b.x);
+                f2_add(hi, lo, make_float2(a.y, b.y));
+                f2_add(hi, lo, make_float2(a.z, b.z));
+                f2_add(hi, lo, make_float2(a.w, b.w));
+            }
+            tot[2 * pp * (FO + 1) + k] = make_float2(hi.x, lo.x);
+            tot[(2 * pp + 1) * (FO + 1) + k] = make_float2(hi.y, lo.y);
+        }
+    } else {
+        for (int q = threadIdx.x; q < FO * NT; q += FT) {
+            const int k = q / NT, t = q % NT, pp = t >> 1, h = t & 1;
+            const T *r = red + k * FT + pp * LY::TP + h;
+            T v = T(0);
+#pragma unroll
+            for (int i = 0; i < LY::TP; i += 2) v += r[i];
+            tot[t * (FO + 1) + k] = v;
+        }
     }
     __syncthreads();
-    if (threadIdx.x < NT) {
-        const int t = threadIdx.x, slot = ly.I * 32 + (int)(blockIdx.x % PARTS) * NT + t;
-        T a[FS], F[3];
-#pragma unroll
-        for (int k = 0; k < FS; ++k) a[k] = tot[t * (FS + 1) + k];
-        own_force<T>(a, own_poles<T>(src, slot, pc.n), F);
-        const double f = fconst, g = fconst / 3;
-        for (int c = 0; c < 3; ++c) {
-            store_acc<double>(frc + (size_t)c * n_pad + slot, -f * (double)F[c], fixed);
-            store_acc<double>(gdip + (size_t)c * n_pad + slot, f * (double)a[c], fixed);
+    // a warp each for the components of the force, and one for the torque sources
+    const int t = threadIdx.x & 31, part = threadIdx.x >> 5;
+    if (t < NT) {
+        const int slot = ly.I * 32 + (int)(blockIdx.x % PARTS) * NT + t;
+        const Vt *a = tot + t * (FO + 1);
+        if (part < 3) {
+            const OwnPoles<T> m = own_poles<T>(src, slot, pc.n);
+            double F;
+            if constexpr (W == 2)
+                F = part == 0 ? own_force_wide<0>(a, m) : part == 1 ? own_force_wide<1>(a, m) : own_force_wide<2>(a, m);
+            else
+                F = part == 0 ? own_force<0>(a, m) : part == 1 ? own_force<1>(a, m) : own_force<2>(a, m);
+            store_acc<double>(frc + (size_t)part * n_pad + slot, -fconst * F, fixed);
+        } else {
+            const int at[6] = {3, 6, 7, 4, 8, 5};   // E_ab: xx xy xz yy yz zz, the diagonal's halved
+            auto value = [&](int k) {
+                if constexpr (W == 2) return f2d_exact(a[k].x) + f2d_exact(a[k].y);
+                else return a[k];
+            };
+            for (int c = 0; c < 3; ++c) store_acc<double>(gdip + (size_t)c * n_pad + slot, fconst * value(c), fixed);
+            for (int c = 0; c < 6; ++c)
+                store_acc<double>(gquad + (size_t)c * n_pad + slot, fconst * (c == 0 || c == 3 || c == 5 ? 2.0 / 3.0 : 1.0 / 3.0) * value(at[c]), fixed);
         }
-        const T Q[6] = {2 * a[3], a[6], a[7], 2 * a[4], a[8], 2 * a[5]};   // xx xy xz yy yz zz
-        for (int c = 0; c < 6; ++c) store_acc<double>(gquad + (size_t)c * n_pad + slot, g * (double)Q[c], fixed);
     }
     if constexpr (VIR) {
         double v[9];
 #pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            double t = (double)Vec<T>::get(vs[k], 0);
-            if (W == 2) t += (double)Vec<T>::get(vs[k], 1);
-            v[k] = 0.5 * fconst * t;
-        }
+        for (int k = 0; k < 9; ++k) v[k] = 0.5 * fconst * vsum[k];
         if (fixed) {
             long long vf[9];
 #pragma unroll
@@ -647,7 +738,7 @@ int pair_forces_p(ap_ctx *ctx, cudaStream_t s, const PoleArgs<T> &src, double *f
     auto kern = vir ? k_pair_forces<T, PARTS, true> : k_pair_forces<T, PARTS, false>;
     // the candidates' rows, or the reduction of the sums
     const size_t bytes = std::max(5 * (AP_CHUNK + 1) * sizeof(typename V4<T>::type),
-                                  sizeof(T) * (Vec<T>::W * FS * FT + 32 * (FS + 1)));
+                                  sizeof(T) * Vec<T>::W * FO * FT + sizeof(double) * 32 * (FO + 1));
     AP_CUDA(allow_smem(kern, bytes));
     kern<<<ctx->n_blocks * PARTS, FT, bytes, s>>>(list_args(ctx), src, frc, gdip, gquad, ctx->n_pad, make_consts<T>(ctx),
                                                   AP_COULOMB, vir, ctx->fixed);

@@ -237,7 +237,21 @@ __device__ __forceinline__ void f2_add(F2 &a, float x) {
     a.lo += (a.hi - (t - z)) + (x - z);
     a.hi = t;
 }
-
+__device__ __forceinline__ float add2(float a, float b) { return a + b; }
+__device__ __forceinline__ float sub2(float a, float b) { return a - b; }
+// the same for float2s (two sums at once) and floats, adding hi + lo of another such sum
+template <class V>
+__device__ __forceinline__ void f2_merge(V &hi, V &lo, V ohi, V olo) {
+    const V t = add2(hi, ohi), z = sub2(t, hi), err = add2(sub2(hi, sub2(t, z)), sub2(ohi, z));
+    lo = add2(add2(lo, olo), err);
+    hi = t;
+}
+template <class V>
+__device__ __forceinline__ void f2_add(V &hi, V &lo, V x) {
+    const V t = add2(hi, x), z = sub2(t, hi);
+    lo = add2(lo, add2(sub2(hi, sub2(t, z)), sub2(x, z)));
+    hi = t;
+}
 
 // A target's sum to its accumulator slot: FP64, or (fixed) 64-bit fixed point. Every slot is
 // written by one thread, from sums formed in a fixed order, so both are reproducible.

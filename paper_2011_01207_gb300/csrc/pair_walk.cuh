@@ -7,7 +7,10 @@
 // each holds both targets in the halves of two-vectors, in FP64 one of them, and walks its share
 // of the pair's list: one shared-memory read of a source serves two pairs, and the whole
 // evaluation is packed. Nobody else adds to these targets, so their sums stay in registers and
-// are stored once: no atomics, no clearing, a fixed order.
+// are stored once: no atomics, no clearing, a fixed order. In FP32 a thread's share of a pair's list (about
+// 22 entries of 175 in water at r_c = 7 A) is summed in FP32, and the threads' shares in compensated FP32 pairs.
+// (Sums in FP64 from the first entry on change the errors against 64 bits by less than 2 %: those of the
+// pairs' own terms are ten times what the sums add.)
 //
 // A list entry is 16 bits: the candidate's place in shared memory (bits 4-15) and four flags for
 // the two targets: excluded pair (bits 0, 1), the target itself (bits 2, 3). An entry stands for
@@ -92,24 +95,45 @@ struct Layout {
         first = W == 2 ? s : s >> 1;         // its first word of the list
     }
     __device__ __forceinline__ int slot() const { return I * 32 + 2 * p + h; }
-    // sum over the threads that share the targets
-    __device__ __forceinline__ typename Vec<T>::type sum(typename Vec<T>::type v) const {
-#pragma unroll
-        for (int off = W == 2 ? 1 : 2; off < TP; off <<= 1) v = add2(v, shfl_xor(v, off));
-        return v;
-    }
-    static __device__ __forceinline__ float2 shfl_xor(float2 v, int off) {
-        return make_float2(__shfl_xor_sync(0xffffffffu, v.x, off), __shfl_xor_sync(0xffffffffu, v.y, off));
-    }
-    static __device__ __forceinline__ double shfl_xor(double v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); }
-    // f[3] summed over the pair's threads, to acc [3][n_pad]
+    // f[3] summed over the threads that share the targets, to acc [3][n_pad]. In FP32 the sums over the
+    // threads are compensated (a thread's own share of a list is a plain FP32 sum). Neighbours share them out: the
+    // target by bit 0 of s, the component by bits 1 and 2 (x, y, then z twice).
     __device__ __forceinline__ void store3(double *__restrict__ acc, int n_pad, const typename Vec<T>::type *f,
                                            int fixed) const {
-        const typename Vec<T>::type a = sum(f[0]), b = sum(f[1]), c = sum(f[2]);
-        // a thread stores component k of target t
-        const int k = W == 2 ? s % 3 : s >> 1, t = W == 2 ? s / 3 : h;
-        const T v = Vec<T>::get(k == 0 ? a : k == 1 ? b : c, t);
-        if (k < 3 && t < 2) store_acc<T>(acc + (size_t)k * n_pad + I * 32 + 2 * p + t, v, fixed);
+        const bool b0 = s & 1, b1 = s & 2, b2 = s & 4;
+        const int t = s & 1;
+        auto shfl = [](auto v, int off) { return __shfl_xor_sync(0xffffffffu, v, off); };
+        if constexpr (W == 2) {
+            float hi[3], lo[3];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                hi[c] = b0 ? f[c].y : f[c].x;
+                lo[c] = 0.f;
+                f2_add(hi[c], lo[c], shfl(b0 ? f[c].x : f[c].y, 1));
+            }
+            float vh = b1 ? hi[2] : hi[0], vl = b1 ? lo[2] : lo[0];
+            f2_merge(vh, vl, shfl(b1 ? hi[0] : hi[2], 2), shfl(b1 ? lo[0] : lo[2], 2));
+            f2_merge(hi[1], lo[1], shfl(hi[1], 2), shfl(lo[1], 2));
+            const bool give = !b1 && !b2, keep = !b1 && b2;   // y goes to the threads with bit 2
+            const float oh = shfl(give ? hi[1] : vh, 4), ol = shfl(give ? lo[1] : vl, 4);
+            if (keep) {
+                vh = hi[1];
+                vl = lo[1];
+            }
+            f2_merge(vh, vl, oh, ol);
+#pragma unroll
+            for (int off = 8; off < TP; off <<= 1) f2_merge(vh, vl, shfl(vh, off), shfl(vl, off));
+            if (s < 8 && !(b1 && b2))
+                store_acc<double>(acc + (size_t)(b1 ? 2 : b2 ? 1 : 0) * n_pad + I * 32 + 2 * p + t, f2d_exact(vh) + f2d_exact(vl), fixed);
+        } else {
+            double a[3] = {f[0], f[1], f[2]};
+#pragma unroll
+            for (int off = 2; off < TP; off <<= 1)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) a[c] += shfl(a[c], off);
+            const int k = s >> 1;   // a thread stores component k of target t
+            if (k < 3) store_acc<double>(acc + (size_t)k * n_pad + I * 32 + 2 * p + t, k == 0 ? a[0] : k == 1 ? a[1] : a[2], fixed);
+        }
     }
 };
 

@@ -1,7 +1,7 @@
 // a2 / a5 - Real-space pair kernels over blocks of 32 atoms (paper Sec. 2.3: groups of B_size
 // atoms with the paper's group-to-atom list filtering). One CTA per block walks the lists of
-// its target pairs (pair_walk.cuh); pair arithmetic in T (FP32 in the mixed and fixed modes), a
-// target's sum in T over its eight threads' shares, stored once as FP64 (or fixed point).
+// its target pairs (pair_walk.cuh); pair arithmetic and a thread's sums in T (FP32 in the mixed and fixed
+// modes), the sum over a target's threads compensated in FP32, stored once as FP64 (or fixed point).
 //
 // Bound by instruction issue (63 % of the slots busy in the matvec at 96,000 atoms, FMA pipe 36 %,
 // shared memory 35 %). Measured on GB300, ncu, warm caches, against the kernels on 32 x 32 pair
