@@ -15,6 +15,7 @@
 // Grid layout: [z][y][x], x contiguous; complex half grid [z][y][x/2+1].
 #include "common.cuh"
 #include "pair_math.cuh"   // packed fma2
+#include "rules.h"
 
 #include <algorithm>
 #include <climits>
@@ -787,9 +788,7 @@ int gather_launch(ap_ctx *ctx, const T *phi, T *out, cudaStream_t s) {
     PmeConsts<T> pc = pme_consts<T>(ctx);
     const int th = ctx->tune_pme_threads;
     const bool wide = sizeof(T) == 4 && ctx->K[0] % 4 == 0;
-    // five threads per atom while they make at most one wave of the GPU's thread slots (wide, one -> five: 9.8
-    // -> 6.1 us at 648 atoms, 10.0 -> 7.9 at 12,288, 11.9 -> 11.1 at 22,969; 14.2 -> 21.2 at 96,000)
-    if (5L * ctx->n <= 2048L * ctx->sm_count) {
+    if (gather_five(ctx->n, ctx->sm_count, ctx->fixed)) {
         auto kern = wide ? k_gather_field5<T, true> : k_gather_field5<T, false>;
         kern<<<lane5_blocks(ctx->n, th), th, 0, s>>>(ctx->stb, (const T4 *)ctx->stw, phi, out, ctx->n_pad, pc);
     } else {
