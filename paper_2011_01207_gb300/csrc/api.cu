@@ -122,6 +122,7 @@ int create_impl(ap_ctx *ctx, const ap_params *P, void *stream) {
     if ((r = dalloc(ctx, &ctx->mlp_feat, sizeof(float) * 16 * np))) return r;
     if ((r = dalloc(ctx, &ctx->mlp_y, sizeof(float) * 3 * np))) return r;
     if ((r = dalloc(ctx, &ctx->e1s, sizeof(double) * 3 * np))) return r;
+    if ((r = lists_init(ctx)) || (r = real_init(ctx)) || (r = forces_init(ctx)) || (r = md_init(ctx))) return r;
     if ((r = pme_init(ctx))) return r;
     AP_CUDA(cudaDeviceSynchronize());
     return AP_OK;

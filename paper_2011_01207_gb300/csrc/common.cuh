@@ -217,11 +217,15 @@ int cfg_load(ap_ctx *ctx, const double *d_xyz, const double *d_mpole, const int 
              const double *d_alpha);
 int lists_launch(ap_ctx *ctx, cudaStream_t s);   // pair lists of the loaded configuration
 int lists_alloc(ap_ctx *ctx);
+// when a context is made: the shared-memory limits of the kernels it launches (allow_smem in pair_walk.cuh)
+int lists_init(ap_ctx *ctx);
+int real_init(ap_ctx *ctx);
+int forces_init(ap_ctx *ctx);
+int md_init(ap_ctx *ctx);
 int real_field_launch(ap_ctx *ctx, cudaStream_t s);
 int real_matvec_launch(ap_ctx *ctx, const void *p, cudaStream_t s);
 int real_matvec_resident_per_sm(ap_ctx *ctx);
 int short_matvec_launch(ap_ctx *ctx, const void *p, double *out, cudaStream_t s);
-int real_forces_launch(ap_ctx *ctx, cudaStream_t s);
 int pme_init(ap_ctx *ctx);
 bool fft_supported(const ap_ctx *ctx);
 int fft_init(ap_ctx *ctx, const float *green);

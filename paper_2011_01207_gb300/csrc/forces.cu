@@ -729,6 +729,21 @@ __global__ void k_unsort3_fx(const double *__restrict__ src, int n_pad, const in
     for (int c = 0; c < 3; ++c) out[3 * i + c] = acc_value(src, (size_t)c * n_pad + s, 1);
 }
 
+// the candidates' rows, or the reduction of the sums
+template <class T>
+constexpr size_t pair_forces_bytes() {
+    return std::max(5 * (AP_CHUNK + 1) * sizeof(typename V4<T>::type),
+                    sizeof(T) * Vec<T>::W * FO * FT + sizeof(double) * 32 * (FO + 1));
+}
+template <class T, int PARTS>
+int init_p(ap_ctx *ctx) {
+    AP_CUDA(allow_smem(k_pair_forces<T, PARTS, false>, pair_forces_bytes<T>()));
+    AP_CUDA(allow_smem(k_pair_forces<T, PARTS, true>, pair_forces_bytes<T>()));
+    return AP_OK;
+}
+template <class T>
+int init_t(ap_ctx *ctx) { return quarter_blocks(ctx) ? init_p<T, 4>(ctx) : init_p<T, 1>(ctx); }
+
 // the real-space force kernel over the current pair lists with the dipoles in ctx->p and the
 // multipoles (dipd, quad0, quad1) given, written to frc, gdip and gquad; with vir given, also the
 // pairs' virial added to vir[0..8]
@@ -736,10 +751,7 @@ template <class T, int PARTS>
 int pair_forces_p(ap_ctx *ctx, cudaStream_t s, const PoleArgs<T> &src, double *frc, double *gdip, double *gquad,
                   double *vir) {
     auto kern = vir ? k_pair_forces<T, PARTS, true> : k_pair_forces<T, PARTS, false>;
-    // the candidates' rows, or the reduction of the sums
-    const size_t bytes = std::max(5 * (AP_CHUNK + 1) * sizeof(typename V4<T>::type),
-                                  sizeof(T) * Vec<T>::W * FO * FT + sizeof(double) * 32 * (FO + 1));
-    AP_CUDA(allow_smem(kern, bytes));
+    const size_t bytes = pair_forces_bytes<T>();
     kern<<<ctx->n_blocks * PARTS, FT, bytes, s>>>(list_args(ctx), src, frc, gdip, gquad, ctx->n_pad, make_consts<T>(ctx),
                                                   AP_COULOMB, vir, ctx->fixed);
     AP_CUDA(cudaGetLastError());
@@ -859,6 +871,8 @@ __global__ void k_virial_out(const double *__restrict__ a, const double *__restr
 }
 
 }  // namespace
+
+int forces_init(ap_ctx *ctx) { return ctx->prec == AP_FP64 ? init_t<double>(ctx) : init_t<float>(ctx); }
 
 int pair_forces_launch(ap_ctx *ctx, cudaStream_t s) {
     return ctx->prec == AP_FP64

@@ -397,7 +397,6 @@ int lists_t(ap_ctx *ctx, cudaStream_t s) {
     // a 1e-5 margin over r_c^2: the walks decide each pair, rounding here drops none
     const T rc2 = (T)(P.cutoff * P.cutoff * (1.0 + 1e-5)), rs2 = (T)(AP_SHORT_RANGE * AP_SHORT_RANGE * (1.0 + 1e-5));
     auto kern = ctx->image_dims ? k_pair_lists<T, true> : k_pair_lists<T, false>;
-    AP_CUDA(allow_smem(kern, sizeof(ListSmem<T>)));
     kern<<<ctx->n_blocks, LT, sizeof(ListSmem<T>), s>>>(ctx->tiles, ctx->tile_off, ctx->excl_mask, (const T4 *)ctx->posw,
                                                         ctx->n, rc2, rs2, (T)P.box[0], (T)P.box[1], (T)P.box[2],
                                                         ctx->image_dims, ctx->list_mult, ctx->ncand, (T4 *)ctx->cand_pos,
@@ -407,7 +406,16 @@ int lists_t(ap_ctx *ctx, cudaStream_t s) {
     return AP_OK;
 }
 
+template <class T>
+int init_t(ap_ctx *ctx) {
+    AP_CUDA(allow_smem(k_pair_lists<T, true>, sizeof(ListSmem<T>)));
+    AP_CUDA(allow_smem(k_pair_lists<T, false>, sizeof(ListSmem<T>)));
+    return AP_OK;
+}
+
 }  // namespace
+
+int lists_init(ap_ctx *ctx) { return ctx->prec == AP_FP64 ? init_t<double>(ctx) : init_t<float>(ctx); }
 
 int lists_launch(ap_ctx *ctx, cudaStream_t s) {
     return ctx->prec == AP_FP64 ? lists_t<double>(ctx, s) : lists_t<float>(ctx, s);

@@ -250,6 +250,9 @@ __global__ void k_add_unsort3(const double *__restrict__ acc, const int *__restr
 }
 
 template <class T>
+constexpr size_t lj_bytes() { return (size_t)(AP_CHUNK + 1) * (sizeof(typename V4<T>::type) + 2 * sizeof(T) + sizeof(int)); }
+
+template <class T>
 int lj_t(ap_ctx *ctx, const double *d_lj, double *d_energy, double *d_forces) {
     typedef typename V4<T>::type T4;
     cudaStream_t s = ctx->s0;
@@ -257,9 +260,7 @@ int lj_t(ap_ctx *ctx, const double *d_lj, double *d_energy, double *d_forces) {
     double *acc = ctx->qv;   // scratch [3][n_pad] (the PCG's q vector, free between solves)
     AP_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * 3 * ctx->n_pad, s));
     AP_CUDA(cudaMemsetAsync(d_energy, 0, sizeof(double), s));
-    const size_t bytes = (size_t)(AP_CHUNK + 1) * (sizeof(T4) + 2 * sizeof(T) + sizeof(int));
-    AP_CUDA(allow_smem(k_lj_forces<T>, bytes));
-    k_lj_forces<T><<<ctx->n_blocks, 128, bytes, s>>>(list_args(ctx), (const T4 *)ctx->posw, ctx->perm, d_lj, ctx->n, ctx->n_pad, (T)P.cutoff, acc, d_energy);
+    k_lj_forces<T><<<ctx->n_blocks, 128, lj_bytes<T>(), s>>>(list_args(ctx), (const T4 *)ctx->posw, ctx->perm, d_lj, ctx->n, ctx->n_pad, (T)P.cutoff, acc, d_energy);
     AP_CUDA(cudaGetLastError());
     k_add_unsort3<<<ap_grid_for(ctx->n, 256), 256, 0, s>>>(acc, ctx->iperm, ctx->n, ctx->n_pad, d_forces);
     AP_CUDA(cudaGetLastError());
@@ -273,6 +274,11 @@ bool lengths_ok(const double *h) {
 }
 
 }  // namespace
+
+int md_init(ap_ctx *ctx) {
+    AP_CUDA(ctx->prec == AP_FP64 ? allow_smem(k_lj_forces<double>, lj_bytes<double>()) : allow_smem(k_lj_forces<float>, lj_bytes<float>()));
+    return AP_OK;
+}
 
 extern "C" int ap_lj_forces(ap_ctx *ctx, const double *d_lj, double *d_energy, double *d_forces) {
     if (!ctx) return AP_ERR_ARG;

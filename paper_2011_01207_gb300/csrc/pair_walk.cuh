@@ -310,7 +310,9 @@ __device__ __forceinline__ void for_chunks(unsigned char *raw, const ListArgs &l
 constexpr int PARTS_BLOCKS = 304;
 inline bool quarter_blocks(const ap_ctx *ctx) { return ctx->n_blocks <= PARTS_BLOCKS; }
 
-// dynamic shared memory above 48 KB has to be asked for once per kernel and device
+// Dynamic shared memory above 48 KB has to be asked for. The limit is the kernel's on its device, shared by every
+// context, so each kernel's is set when a context is made, to the most that any launch can need: set before a launch
+// to what that one needs, it could be lowered by another thread's before the launch came.
 template <class K>
 inline cudaError_t allow_smem(K kernel, size_t bytes) {
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);

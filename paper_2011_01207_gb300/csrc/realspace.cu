@@ -146,7 +146,6 @@ int perm_field_t(ap_ctx *ctx, cudaStream_t s) {
     typedef typename V4<T>::type T4;
     auto kern = k_perm_field<T, PARTS>;
     const size_t bytes = rows_bytes<T>(4);
-    AP_CUDA(allow_smem(kern, bytes));
     kern<<<ctx->n_blocks * PARTS, PT, bytes, s>>>(list_args(ctx), (const T4 *)ctx->posw, (const T4 *)ctx->dipd,
                                                   (const T4 *)ctx->quad0, (const T4 *)ctx->quad1, ctx->acc, ctx->n_pad,
                                                   make_consts<T>(ctx), ctx->fixed);
@@ -167,7 +166,6 @@ int matvec_p(ap_ctx *ctx, const void *p0, const void *p1, double *acc0, double *
     typedef typename V4<T>::type T4;
     auto kern = k_matvec<T, PARTS, NS, SHORT>;
     const size_t bytes = matvec_bytes(rows_bytes<T>(1 + NS), NS == 1 && !SHORT ? ctx->tune_mv_per_sm : 0);
-    AP_CUDA(allow_smem(kern, bytes));
     kern<<<ctx->n_blocks * PARTS, PT, bytes, s>>>(list_args(ctx), (const T4 *)ctx->posw, (const T4 *)p0, (const T4 *)p1, acc0,
                                                   acc1, ctx->n_pad, make_consts<T>(ctx), ctx->fixed);
     AP_CUDA(cudaGetLastError());
@@ -183,9 +181,23 @@ template <class T>
 int resident_t() {
     int per_sm = 0;
     const size_t bytes = rows_bytes<T>(2);
-    allow_smem(k_matvec<T, 1, 1, false>, bytes);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_matvec<T, 1, 1, false>, PT, bytes);
     return std::max(1, per_sm);
+}
+
+template <class T, int PARTS>
+int init_p(ap_ctx *ctx) {
+    AP_CUDA(allow_smem(k_perm_field<T, PARTS>, rows_bytes<T>(4)));
+    AP_CUDA(allow_smem(k_matvec<T, PARTS, 1, false>, SM_SMEM));   // whatever the autotuner chooses
+    AP_CUDA(allow_smem(k_matvec<T, PARTS, 1, true>, rows_bytes<T>(2)));
+    AP_CUDA(allow_smem(k_matvec<T, PARTS, 2, false>, rows_bytes<T>(3)));
+    return AP_OK;
+}
+template <class T>
+int init_t(ap_ctx *ctx) {
+    // (the count of resident CTAs is always the whole-block kernel's)
+    AP_CUDA(allow_smem(k_matvec<T, 1, 1, false>, SM_SMEM));
+    return quarter_blocks(ctx) ? init_p<T, 4>(ctx) : init_p<T, 1>(ctx);
 }
 
 template <class T>
@@ -194,6 +206,8 @@ int field_t(ap_ctx *ctx, cudaStream_t s) {
 }
 
 }  // namespace
+
+int real_init(ap_ctx *ctx) { return ctx->prec == AP_FP64 ? init_t<double>(ctx) : init_t<float>(ctx); }
 
 int short_matvec_launch(ap_ctx *ctx, const void *p, double *out, cudaStream_t s) {
     return ctx->prec == AP_FP64 ? matvec_t<double, 1, true>(ctx, p, nullptr, out, nullptr, s)
