@@ -33,7 +33,7 @@ void free_all(ap_ctx *c) {
                     c->grid, c->cgrid, c->cgrid_v, c->green, c->grid2, c->frc, c->gdip, c->gquad, c->red, c->mu_s, c->gbuf,
                     c->tile_off, c->ncand, c->cand_j, c->cand_pos, c->cand_mask, c->list, c->list_meta,
                     c->red_part, c->mlp_feat, c->mlp_y, c->e1s, c->dg, c->stb, c->stw, c->grid_fx,
-                    c->hist_count, c->mu_f, c->r_f, c->q_f, c->dga_f, c->bhalf, c->nb_info, c->fft_tw, c->fft_green};
+                    c->hist_count, c->mu_f, c->r_f, c->q_f, c->dga_f, c->bhalf, c->nb_info, c->boxes, c->fft_tw, c->fft_green};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     diis_release(c);
@@ -78,6 +78,7 @@ int create_impl(ap_ctx *ctx, const ap_params *P, void *stream) {
     if ((r = dalloc(ctx, &ctx->tile_off, sizeof(int) * (nb + 1)))) return r;
     if ((r = dalloc(ctx, &ctx->bhalf, sizeof(float4) * nb))) return r;
     if ((r = dalloc(ctx, &ctx->nb_info, sizeof(int) * 8))) return r;
+    if ((r = dalloc(ctx, (char **)&ctx->boxes, 8 * es * nb))) return r;
     if ((r = dalloc(ctx, (char **)&ctx->posq, 4 * es * np))) return r;
     if ((r = dalloc(ctx, (char **)&ctx->posw, 4 * es * np))) return r;
     if ((r = dalloc(ctx, &ctx->stb, sizeof(int4) * np))) return r;

@@ -99,6 +99,7 @@ struct ap_ctx {
     int image_dims = 0;          // bit d: the box is too short along d for one image per tile
     // pair lists of the configuration (lists.cu, walked as in pair_walk.cuh)
     int list_mult = 1;           // images an atom can appear in beside one block (2 per short dimension)
+    void *boxes = nullptr;       // T4 [n_blocks][2] centres and half extents at the present positions
     int4 *ncand = nullptr;       // [n_blocks] candidate atoms in the block's four segments
     int *cand_j = nullptr;       // [cap][32] candidate's slot | AP_CAND_SELF
     void *cand_pos = nullptr;    // T4 [cap][32] candidate's position beside the block, Thole factor

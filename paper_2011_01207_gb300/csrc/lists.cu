@@ -13,7 +13,8 @@
 // no kernel adds into another's targets. (On masks, half of a kernel's time went into staging and
 // flushing items of 32 x 32 slots with 124 pairs in them.)
 //
-// One CTA per block. Each of its four warps takes a contiguous quarter of the block's tiles:
+// One CTA per block. Each of its four warps takes every fourth of the block's tiles (a contiguous quarter
+// each left the CTA waiting for the warps with the nearest blocks, a sixth of its time):
 // atoms that pass the bounding-box test queue up, and every 32 of them are tested against the
 // block's atoms, a lane holding one candidate and reading the targets from shared memory (in FP32
 // two at a time, packed, the sign of r^2 - r_c^2 shifted into the candidate's word); the result is
@@ -21,8 +22,11 @@
 // per target pair, whose set bits eight threads per pair count and write out as entries, through shared memory so that the list goes out in whole lines.
 // Measured on GB300 (ncu, warm) against filtered chunks, pair masks and work-item scans (k_filter,
 // k_pairmask and five small kernels): 96,000 atoms 76 + 42 + 17 -> 137 us in one launch, 6,000 atoms
-// (short box) 342 + 20 + 15 -> 55 us; the kernels that walk the lists gain 40 % and more. Bound by
-// issue and latency together (50 % of the slots, 5 CTAs per SM).
+// (short box) 342 + 20 + 15 -> 55 us; the kernels that walk the lists gain 40 % and more. That took longer in
+// permanent_field alone above 200,000 atoms, where nothing hides it: 693 -> 724 us at 255,552, 1,613 -> 1,752 at 648,000,
+// 2,700 -> 2,936 at 1,065,000. Interleaved tiles, entries written without a search for bits, a look at whole blocks
+// first, and two tiles in flight instead of four (64 registers, 8 CTAs an SM instead of 5: it is bound by issue and
+// latency together, 55 % of the slots at 5) made those 605, 1,443 and 2,431.
 // Candidate and entry order follow the tile order, so the lists are the same in every run.
 #include "common.cuh"
 #include "pair_walk.cuh"
@@ -133,13 +137,42 @@ __device__ __forceinline__ unsigned warp_transpose32(unsigned x, int lane) {
     return x;
 }
 
+// The blocks' boxes at their atoms' present places: centre (relative to the block's origin) and half extents, a
+// little more than the atoms reach. One warp a block.
+template <class T>
+__global__ void k_boxes(const typename V4<T>::type *__restrict__ posw, int n_atoms, int n_blocks,
+                        typename V4<T>::type *__restrict__ boxes) {
+    const int b = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (b >= n_blocks) return;
+    const typename V4<T>::type me = posw[b * 32 + lane];
+    const bool real = b * 32 + lane < n_atoms;
+    const T x[3] = {me.x, me.y, me.z};
+    T c[3], h[3];
+    for (int d = 0; d < 3; ++d) {
+        T lo = real ? x[d] : T(1e30), hi = real ? x[d] : T(-1e30);
+        for (int off = 16; off; off >>= 1) {
+            lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, off));
+            hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, off));
+        }
+        c[d] = T(0.5) * (lo + hi);
+        h[d] = T(0.5) * (hi - lo) + T(1e-6) * max(abs(lo), abs(hi));
+    }
+    if (lane == 0) {
+        typename V4<T>::type v;
+        v.x = c[0]; v.y = c[1]; v.z = c[2]; v.w = T(0);
+        boxes[2 * b] = v;
+        v.x = h[0]; v.y = h[1]; v.z = h[2];
+        boxes[2 * b + 1] = v;
+    }
+}
+
 // dims: bit d set where the box is so short along d that an atom may be in range of one block in
 // two images (IMAGES: any); a tile's atoms are then taken in the image nearest the block and its
 // neighbours along those dimensions
 template <class T, bool IMAGES>
-__global__ void __launch_bounds__(LT, 5) k_pair_lists(
+__global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_lists(
     const TileRec *__restrict__ tiles, const int *__restrict__ tile_off, const unsigned *__restrict__ excl_mask,
-    const typename V4<T>::type *__restrict__ posw, int n_atoms, T rc2, T rs2, T Lx, T Ly, T Lz, int dims, int mult,
+    const typename V4<T>::type *__restrict__ posw, const typename V4<T>::type *__restrict__ boxes, int n_atoms, T rc2, T rs2, T Lx, T Ly, T Lz, int dims, int mult,
     int4 *__restrict__ ncand, typename V4<T>::type *__restrict__ cand_pos, int *__restrict__ cand_j,
     uint4 *__restrict__ cand_mask, uint2 *__restrict__ meta, unsigned short *__restrict__ list) {
     typedef typename V4<T>::type T4;
@@ -160,12 +193,11 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
         ctr[d] = T(0.5) * (lo + hi);
         half[d] = T(0.5) * (hi - lo) * T(1.0 + 1e-6);   // not less than the targets reach
     }
-    const int t0 = tile_off[I], nt = tile_off[I + 1] - t0, share = (nt + 3) >> 2;
-    const int tb = t0 + min(w * share, nt), te = t0 + min((w + 1) * share, nt);
+    const int t0 = tile_off[I], nt = tile_off[I + 1] - t0, te = t0 + nt;
     __syncthreads();
 
-    const size_t seg = (size_t)tb * 32 * mult;
-    const int room = (te - tb) * 32 * mult;
+    const size_t seg = ((size_t)t0 + segment_tile(nt, w)) * 32 * mult;
+    const int room = (segment_tile(nt, w + 1) - segment_tile(nt, w)) * 32 * mult;
     int queued = 0, kept = 0;
     auto push = [&](T x, T y, T z, T wt, int j, unsigned ex, bool ok) {
         const T gx = max(T(0), abs(x - ctr[0]) - half[0]);
@@ -173,6 +205,7 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
         const T gz = max(T(0), abs(z - ctr[2]) - half[2]);
         const bool sel = ok && gx * gx + gy * gy + gz * gz < rc2;
         const unsigned b = __ballot_sync(0xffffffffu, sel);
+        if (!b) return;   // a third of the tiles: lists are kept for cutoff + buffer
         if (sel) {
             const int k = queued + __popc(b & ((1u << lane) - 1u));
             T4 v;
@@ -195,61 +228,82 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
             __syncwarp();
         }
     };
-    // four tiles' loads go out together: the loop waits for memory, not for arithmetic
-    constexpr int U = 4;
-    for (int tr = tb; tr < te; tr += U) {
-        TileRec rec[U];
-        T4 qv[U];
-        unsigned ev[U];
+    // With the boxes at hand a lane looks at one of the warp's tiles each, and those whose blocks are out of range
+    // as a whole (a third: the list of tiles is made for cutoff + buffer) go no further.
+    for (int base = t0 + w; base < te; base += 4 * 32) {
+        const int mine = base + 4 * lane;
+        bool near_block = mine < te;
+        if (!IMAGES && boxes && near_block) {
+            const TileRec t = tiles[mine];
+            const T4 bc = boxes[2 * t.J], bh = boxes[2 * t.J + 1];
+            const T gx = max(T(0), abs((bc.x + (T)t.lx) + (T)t.hx - ctr[0]) - half[0] - bh.x);
+            const T gy = max(T(0), abs((bc.y + (T)t.ly) + (T)t.hy - ctr[1]) - half[1] - bh.y);
+            const T gz = max(T(0), abs((bc.z + (T)t.lz) + (T)t.hz - ctr[2]) - half[2] - bh.z);
+            near_block = gx * gx + gy * gy + gz * gz < rc2;
+        }
+        unsigned todo = __ballot_sync(0xffffffffu, near_block);
+        // two tiles' loads go out together (four would take the registers of three CTAs an SM)
+        constexpr int U = 2;
+        while (todo) {
+            TileRec rec[U];
+            int tr[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (tr + u < te) rec[u] = tiles[tr + u];
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (tr + u < te) {
-                qv[u] = posw[rec[u].J * 32 + lane];
-                ev[u] = rec[u].excl >= 0 ? excl_mask[(size_t)rec[u].excl * 32 + lane] : 0u;
+            for (int u = 0; u < U; ++u) {
+                tr[u] = todo ? base + 4 * (__ffs(todo) - 1) : te;
+                todo &= todo - 1u;
             }
+            T4 qv[U];
+            unsigned ev[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (tr + u >= te) break;   // uniform over the warp
-            const TileRec &t = rec[u];
-            // positions are relative to their block's origin: moved to block I's origin with the
-            // tile's offset, a float pair (hi + lo), so that the result (a few A) has full FP32
-            // precision at any box size
-            const T x = (qv[u].x + (T)t.lx) + (T)t.hx, y = (qv[u].y + (T)t.ly) + (T)t.hy, z = (qv[u].z + (T)t.lz) + (T)t.hz;
-            const int slot = t.J * 32 + lane;
-            if constexpr (!IMAGES) {
-                push(x, y, z, qv[u].w, t.J == I ? slot | AP_CAND_SELF : slot, ev[u], true);
-            } else {
-                // along a short dimension: the image nearest the box's centre (k0), and the next one on
-                // the other side, each only if it lies within r_c of the box along that dimension
-                const T L[3] = {Lx, Ly, Lz}, rc = sqrt(rc2);
-                T c[3] = {x, y, z}, alt[3];
-                int k0[3] = {0, 0, 0}, k1[3] = {0, 0, 0};
-                bool near[3] = {true, true, true}, far[3] = {false, false, false};
-                const bool real = slot < n_atoms;
+            for (int u = 0; u < U; ++u)
+                if (tr[u] < te) rec[u] = tiles[tr[u]];
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    alt[d] = c[d];
-                    if (((dims >> d) & 1) && real) {
-                        const T k = rint((c[d] - ctr[d]) / L[d]), sgn = c[d] - L[d] * k > ctr[d] ? T(1) : T(-1);
-                        k0[d] = (int)k;
-                        k1[d] = (int)(k + sgn);
-                        c[d] = alt[d] - L[d] * k;
-                        alt[d] -= L[d] * (k + sgn);
-                        near[d] = abs(c[d] - ctr[d]) - half[d] < rc;
-                        far[d] = abs(alt[d] - ctr[d]) - half[d] < rc;
-                    }
+            for (int u = 0; u < U; ++u)
+                if (tr[u] < te) {
+                    qv[u] = posw[rec[u].J * 32 + lane];
+                    ev[u] = rec[u].excl >= 0 ? excl_mask[(size_t)rec[u].excl * 32 + lane] : 0u;
                 }
-                for (int im = 0; im < 8; ++im) {
-                    if (im & ~dims) continue;   // uniform over the launch
-                    const bool i0 = im & 1, i1 = im & 2, i2 = im & 4;
-                    const bool ok = (i0 ? far[0] : near[0]) && (i1 ? far[1] : near[1]) && (i2 ? far[2] : near[2]);
-                    if (!__any_sync(0xffffffffu, ok)) continue;
-                    const bool own = t.J == I && (i0 ? k1[0] : k0[0]) == 0 && (i1 ? k1[1] : k0[1]) == 0 && (i2 ? k1[2] : k0[2]) == 0;
-                    push(i0 ? alt[0] : c[0], i1 ? alt[1] : c[1], i2 ? alt[2] : c[2], qv[u].w,
-                         own ? slot | AP_CAND_SELF : slot, ev[u], ok);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (tr[u] >= te) break;   // uniform over the warp
+                const TileRec &t = rec[u];
+                // positions are relative to their block's origin: moved to block I's origin with the
+                // tile's offset, a float pair (hi + lo), so that the result (a few A) has full FP32
+                // precision at any box size
+                const T x = (qv[u].x + (T)t.lx) + (T)t.hx, y = (qv[u].y + (T)t.ly) + (T)t.hy, z = (qv[u].z + (T)t.lz) + (T)t.hz;
+                const int slot = t.J * 32 + lane;
+                if constexpr (!IMAGES) {
+                    push(x, y, z, qv[u].w, t.J == I ? slot | AP_CAND_SELF : slot, ev[u], true);
+                } else {
+                    // along a short dimension: the image nearest the box's centre (k0), and the next one on
+                    // the other side, each only if it lies within r_c of the box along that dimension
+                    const T L[3] = {Lx, Ly, Lz}, rc = sqrt(rc2);
+                    T c[3] = {x, y, z}, alt[3];
+                    int k0[3] = {0, 0, 0}, k1[3] = {0, 0, 0};
+                    bool near[3] = {true, true, true}, far[3] = {false, false, false};
+                    const bool real = slot < n_atoms;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        alt[d] = c[d];
+                        if (((dims >> d) & 1) && real) {
+                            const T k = rint((c[d] - ctr[d]) / L[d]), sgn = c[d] - L[d] * k > ctr[d] ? T(1) : T(-1);
+                            k0[d] = (int)k;
+                            k1[d] = (int)(k + sgn);
+                            c[d] = alt[d] - L[d] * k;
+                            alt[d] -= L[d] * (k + sgn);
+                            near[d] = abs(c[d] - ctr[d]) - half[d] < rc;
+                            far[d] = abs(alt[d] - ctr[d]) - half[d] < rc;
+                        }
+                    }
+                    for (int im = 0; im < 8; ++im) {
+                        if (im & ~dims) continue;   // uniform over the launch
+                        const bool i0 = im & 1, i1 = im & 2, i2 = im & 4;
+                        const bool ok = (i0 ? far[0] : near[0]) && (i1 ? far[1] : near[1]) && (i2 ? far[2] : near[2]);
+                        if (!__any_sync(0xffffffffu, ok)) continue;
+                        const bool own = t.J == I && (i0 ? k1[0] : k0[0]) == 0 && (i1 ? k1[1] : k0[1]) == 0 && (i2 ? k1[2] : k0[2]) == 0;
+                        push(i0 ? alt[0] : c[0], i1 ? alt[1] : c[1], i2 ? alt[2] : c[2], qv[u].w,
+                             own ? slot | AP_CAND_SELF : slot, ev[u], ok);
+                    }
                 }
             }
         }
@@ -261,7 +315,7 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
 
     // ---- the lists, chunk by chunk
     const int e1 = S.count[0], e2 = e1 + S.count[1], e3 = e2 + S.count[2], n = e3 + S.count[3];
-    auto seg_start = [&](int q) { return ((size_t)t0 + min(q * share, nt)) * 32 * mult; };
+    auto seg_start = [&](int q) { return ((size_t)t0 + segment_tile(nt, q)) * 32 * mult; };
     const size_t b0 = seg_start(0), b1 = seg_start(1) - e1, b2 = seg_start(2) - e2, b3 = seg_start(3) - e3;
     const int chunks = (n + AP_CHUNK - 1) / AP_CHUNK;
     const int per = chunks ? (n + chunks - 1) / chunks : 0;
@@ -271,12 +325,16 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
     for (int c = 0; c < chunks; ++c) {
         const int k0 = c * per, kc = min(per, n - k0);
         const int groups = (kc + 31) >> 5;
-        for (int g = w; g < groups; g += 4) {
+        auto masks = [&](int g) {
             const int k = g * 32 + lane, kk = k0 + k;
+            const size_t at = (kk < e1 ? b0 : kk < e2 ? b1 : kk < e3 ? b2 : b3) + kk;
+            return k < kc ? cand_mask[at] : make_uint4(0u, 0u, 0u, 0u);
+        };
+        for (int g = w; g < groups; g += 4) {
+            const int k = g * 32 + lane;
+            const uint4 m = masks(g);
             unsigned in = 0u, sh = 0u, ex = 0u, own = 0u;
             if (k < kc) {
-                const size_t at = (kk < e1 ? b0 : kk < e2 ? b1 : kk < e3 ? b2 : b3) + kk;
-                const uint4 m = cand_mask[at];
                 in = m.x;
                 sh = m.y;
                 ex = m.z;
@@ -309,7 +367,7 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
         // beyond the rows of the list fills the holes of the shorter ones, phantoms the last.
         const unsigned cls = 0x01010101u << s;
         int c0 = 0, c1 = 0, c2 = 0;
-        unsigned used[3] = {0u, 0u, 0u};   // the groups with anything of the three kinds in them
+        unsigned used[2] = {0u, 0u};   // the groups with any flagged and any short-range entry
         for (int g = 0; g < groups; ++g) {
             const unsigned a = S.word[0][p][g] & cls, b = S.word[1][p][g] & cls, d = S.word[2][p][g] & cls;
             c0 += __popc(a);
@@ -317,7 +375,6 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
             c2 += __popc(d);
             if (a) used[0] |= 1u << g;
             if (b) used[1] |= 1u << g;
-            if (d) used[2] |= 1u << g;
         }
         const int mine = c0 + c1 + c2;
         int np = mine;
@@ -348,34 +405,52 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
             all += S.total[q];
         }
         const bool staged = all <= STAGE;
-        unsigned short *out = staged ? S.stage + off : list + entries + done + off;
-        auto put = [&](int row, int col, unsigned e) { out[(((row >> 1) * 8 + col) << 1) | (row & 1)] = (unsigned short)e; };
-        int at = 0;
+        auto flags = [&](int k) { return ((S.ex[k] >> (2 * p)) & 3u) | (((S.own[k] >> (2 * p)) & 3u) << 2); };
+        auto emit = [&](unsigned short *out) {
+            auto put = [&](int row, int col, unsigned e) { out[(((row >> 1) * 8 + col) << 1) | (row & 1)] = (unsigned short)e; };
+            // No bits are searched for: the warp goes through the groups that have any of a kind, every thread
+            // looking at its four places in turn.
+            int at = 0;
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            while (used[q]) {
-                const int g = __ffs(used[q]) - 1;
-                used[q] &= used[q] - 1u;
-                unsigned m = S.word[q][p][g] & cls;
-                while (m) {
-                    const int k = g * 32 + __ffs(m) - 1;
-                    m &= m - 1u;
-                    unsigned e = (unsigned)k << 4;
-                    if (q == 0) e |= ((S.ex[k] >> (2 * p)) & 3u) | (((S.own[k] >> (2 * p)) & 3u) << 2);
-                    if (at < rows) {
-                        put(at, s, e);
-                    } else {   // hole number h, in the last column whose holes start at or before it
-                        const int h = po + at - rows;
-                        int col = 7;
-                        while (S.column[p][col].x > h || S.column[p][col].y >= rows) --col;
-                        put(S.column[p][col].y + h - S.column[p][col].x, col, e);
+            for (int q = 0; q < 2; ++q) {
+                while (used[q]) {
+                    const int g = __ffs(used[q]) - 1;
+                    used[q] &= used[q] - 1u;
+                    unsigned m = S.word[q][p][g] & cls;
+                    while (m) {
+                        const int k = g * 32 + __ffs(m) - 1;
+                        m &= m - 1u;
+                        if (at < rows) put(at, s, (unsigned)k << 4 | (q == 0 ? flags(k) : 0u));
+                        ++at;
                     }
-                    ++at;
                 }
             }
-        }
-        for (int k = 0; k < hole; ++k)
-            if (ph + k >= all_over) put(mine + k, s, (unsigned)kc << 4);   // the phantom
+            for (int g = 0; g < groups; ++g) {
+                const unsigned m = S.word[2][p][g] >> s;
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    const bool on = (m >> (8 * b)) & 1u;
+                    if (on && at < rows) put(at, s, (unsigned)(g * 32 + s + 8 * b) << 4);
+                    at += on;
+                }
+            }
+            // what the column has beyond the rows, from the end: hole number h is in the last column whose holes
+            // start at or before it
+            for (int q = 2, left = over; left; --q)
+                for (int g = groups - 1; left && g >= 0; --g) {
+                    unsigned m = S.word[q][p][g] & cls;
+                    for (; left && m; --left) {
+                        const int bit = 31 - __clz(m), k = g * 32 + bit, h = po + left - 1;
+                        m ^= 1u << bit;
+                        int col = 7;
+                        while (S.column[p][col].x > h || S.column[p][col].y >= rows) --col;
+                        put(S.column[p][col].y + h - S.column[p][col].x, col, (unsigned)k << 4 | (q == 0 ? flags(k) : 0u));
+                    }
+                }
+            for (int k = 0; k < hole; ++k)
+                if (ph + k >= all_over) put(mine + k, s, (unsigned)kc << 4);   // the phantom
+        };
+        emit(staged ? S.stage + off : list + entries + done + off);
         if (s == 0)   // where it lies; its rounds of 16 entries, those with flagged and with short-range ones
             meta[metas + (size_t)c * 16 + p] = make_uint2((unsigned)(done + off), (unsigned)rounds |
                                                           ((unsigned)((r0 + 1) >> 1) << 10) | ((unsigned)((r1 + 1) >> 1) << 20));
@@ -390,6 +465,10 @@ __global__ void __launch_bounds__(LT, 5) k_pair_lists(
     }
 }
 
+// Blocks per SM from which the tiles are first tested as a whole, by the blocks' present boxes: as many CTAs as
+// are resident (field, without -> with: 102.2 -> 104.8 us at 750 blocks, 165.0 -> 163.5 at 1,465, 253.4 -> 252.4 at 3,000,
+// 619 -> 602.6 at 7,986; the boxes are a launch of their own, which a system of one wave waits for).
+constexpr int BOXES_MIN = 8;
 template <class T>
 int lists_t(ap_ctx *ctx, cudaStream_t s) {
     typedef typename V4<T>::type T4;
@@ -397,7 +476,12 @@ int lists_t(ap_ctx *ctx, cudaStream_t s) {
     // a 1e-5 margin over r_c^2: the walks decide each pair, rounding here drops none
     const T rc2 = (T)(P.cutoff * P.cutoff * (1.0 + 1e-5)), rs2 = (T)(AP_SHORT_RANGE * AP_SHORT_RANGE * (1.0 + 1e-5));
     auto kern = ctx->image_dims ? k_pair_lists<T, true> : k_pair_lists<T, false>;
-    kern<<<ctx->n_blocks, LT, sizeof(ListSmem<T>), s>>>(ctx->tiles, ctx->tile_off, ctx->excl_mask, (const T4 *)ctx->posw,
+    const T4 *boxes = nullptr;
+    if (ctx->n_blocks >= BOXES_MIN * ctx->sm_count && !ctx->image_dims) {
+        boxes = (const T4 *)ctx->boxes;
+        k_boxes<T><<<ap_grid_for(32L * ctx->n_blocks, 128), 128, 0, s>>>((const T4 *)ctx->posw, ctx->n, ctx->n_blocks, (T4 *)ctx->boxes);
+    }
+    kern<<<ctx->n_blocks, LT, sizeof(ListSmem<T>), s>>>(ctx->tiles, ctx->tile_off, ctx->excl_mask, (const T4 *)ctx->posw, boxes,
                                                         ctx->n, rc2, rs2, (T)P.box[0], (T)P.box[1], (T)P.box[2],
                                                         ctx->image_dims, ctx->list_mult, ctx->ncand, (T4 *)ctx->cand_pos,
                                                         ctx->cand_j, ctx->cand_mask, ctx->list_meta,

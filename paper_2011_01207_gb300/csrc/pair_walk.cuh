@@ -55,16 +55,19 @@ __host__ __device__ __forceinline__ size_t list_meta_base(int tile0, int I, int 
     return ((size_t)tile0 * mult) / (AP_CHUNK / 32) + I;
 }
 
-// the candidates of one block: four segments (one per warp of the list kernel), each starting
-// at its share of the block's tiles
+// Warp w of the list kernel takes every fourth of a block's nt tiles, from tile w on: the first tile of its
+// segment when the warps' tiles are laid one warp after the other
+__host__ __device__ __forceinline__ int segment_tile(int nt, int w) { return w * (nt >> 2) + (w < (nt & 3) ? w : nt & 3); }
+
+// the candidates of one block: four segments (one per warp of the list kernel)
 struct Cands {
     size_t start[4];
     int p1, p2, p3, n;      // ends of the first three segments in the block's order, and the total
     __device__ __forceinline__ Cands(const ListArgs &la, int I) {
-        const int t0 = la.tile_off[I], nt = la.tile_off[I + 1] - t0, q = (nt + 3) >> 2;
+        const int t0 = la.tile_off[I], nt = la.tile_off[I + 1] - t0;
         const int4 c = la.ncand[I];
 #pragma unroll
-        for (int w = 0; w < 4; ++w) start[w] = ((size_t)t0 + min(w * q, nt)) * 32 * la.mult;
+        for (int w = 0; w < 4; ++w) start[w] = ((size_t)t0 + segment_tile(nt, w)) * 32 * la.mult;
         p1 = c.x;
         p2 = p1 + c.y;
         p3 = p2 + c.z;
