@@ -31,7 +31,7 @@ void free_all(ap_ctx *c) {
                     c->tmp_int, c->posq, c->posw, c->dipd, c->quad0, c->quad1, c->alpha,
                     c->E, c->acc, c->rec, c->rot, c->mpl, c->frame_s, c->fvec, c->mu, c->r, c->qv, c->p, c->st,
                     c->grid, c->cgrid, c->cgrid_v, c->green, c->grid2, c->frc, c->gdip, c->gquad, c->red, c->mu_s, c->gbuf,
-                    c->tile_off, c->ncand, c->cand_j, c->cand_pos, c->cand_mask, c->list, c->list_meta,
+                    c->tile_off, c->ncand, c->cand_j, c->cand_pos, c->list, c->list_meta,
                     c->red_part, c->mlp_feat, c->mlp_y, c->e1s, c->dg, c->stb, c->stw, c->grid_fx,
                     c->hist_count, c->mu_f, c->r_f, c->q_f, c->dga_f, c->bhalf, c->nb_info, c->boxes, c->fft_tw, c->fft_green};
     for (void *p : ptrs)

@@ -8,14 +8,11 @@
 #include <string>
 
 #include "../../include/amoebapol.h"
+#include "rules.h"
 
 #define AP_WARP 32
 #define AP_BLOCK_ATOMS 32          // atoms per block, paper Sec. 2.3: B_size = 32
-#define AP_CHUNK 640               // candidate atoms of a block staged in shared memory at once
 #define AP_CAND_SELF (1 << 30)     // a candidate that is an atom of the block itself
-#define AP_LIST_PER_TILE 528       // capacity of the pair lists, entries per tile: 32 candidates x 16 target
-                                   // pairs, and the padding of a chunk's 16 lists spread over its tiles
-#define AP_LIST_PER_BLOCK 256
 
 // physical constants (readings: the paper gives none)
 #define AP_COULOMB 332.063713       // kcal A / (mol e^2)
@@ -103,8 +100,8 @@ struct ap_ctx {
     int4 *ncand = nullptr;       // [n_blocks] candidate atoms in the block's four segments
     int *cand_j = nullptr;       // [cap][32] candidate's slot | AP_CAND_SELF
     void *cand_pos = nullptr;    // T4 [cap][32] candidate's position beside the block, Thole factor
-    uint4 *cand_mask = nullptr;  // [cap][32] in-range, short-range and exclusion bits (bit i-lane), cand_j
-    unsigned *list = nullptr;    // the lists' entries, two per word
+    unsigned *list = nullptr;    // the lists' entries, two per word (while they are made also the candidates'
+                                 // masks: rules.h)
     uint2 *list_meta = nullptr;  // [chunk][16] where each target pair's list lies
     double *e1s = nullptr;       // [3][n_pad] short-range first-order induced field (feature)
     long cap_lists = 0;          // tiles x images the candidate and list arrays hold

@@ -102,11 +102,11 @@ struct ListSmem {
 };
 
 // 32 (or the last m) queued candidates against the block's atoms: the ones in range of any go to
-// the candidate arrays at `at`, of which `room` are left; returns how many
+// the candidate arrays at `at`, of which `room` are left, and their masks to `mask`; returns how many
 template <class T>
 __device__ __forceinline__ int test_queue(const ListSmem<T> &S, int w, int lane, int m, T rc2, T rs2, size_t at, int room,
                                           typename V4<T>::type *__restrict__ cand_pos, int *__restrict__ cand_j,
-                                          uint4 *__restrict__ cand_mask) {
+                                          uint4 *mask) {
     const typename V4<T>::type c = S.q.pos[w][lane];
     const int j = S.q.j[w][lane];
     unsigned in, sh;
@@ -116,10 +116,11 @@ __device__ __forceinline__ int test_queue(const ListSmem<T> &S, int w, int lane,
     const unsigned b = __ballot_sync(0xffffffffu, keep);
     // (rounding at 2 r_c = L could make a third image; the room is for two)
     if (keep && __popc(b & ((1u << lane) - 1u)) < room) {
-        const size_t k = at + __popc(b & ((1u << lane) - 1u));
-        cand_pos[k] = c;
-        cand_j[k] = j;
-        cand_mask[k] = make_uint4(in, sh & in, S.q.ex[w][lane] & in, (unsigned)j);
+        const int k = __popc(b & ((1u << lane) - 1u));
+        cand_pos[at + k] = c;
+        cand_j[at + k] = j;
+        // in-range, short-range and exclusion bits (bit i-lane), and j
+        mask[k] = make_uint4(in, sh & in, S.q.ex[w][lane] & in, (unsigned)j);
     }
     return min(__popc(b), room);
 }
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_
     const TileRec *__restrict__ tiles, const int *__restrict__ tile_off, const unsigned *__restrict__ excl_mask,
     const typename V4<T>::type *__restrict__ posw, const typename V4<T>::type *__restrict__ boxes, int n_atoms, T rc2, T rs2, T Lx, T Ly, T Lz, int dims, int mult,
     int4 *__restrict__ ncand, typename V4<T>::type *__restrict__ cand_pos, int *__restrict__ cand_j,
-    uint4 *__restrict__ cand_mask, uint2 *__restrict__ meta, unsigned short *__restrict__ list) {
+    uint2 *__restrict__ meta, unsigned short *list) {
     typedef typename V4<T>::type T4;
     extern __shared__ __align__(16) unsigned char raw[];
     ListSmem<T> &S = *reinterpret_cast<ListSmem<T> *>(raw);
@@ -197,6 +198,8 @@ __global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_
     __syncthreads();
 
     const size_t seg = ((size_t)t0 + segment_tile(nt, w)) * 32 * mult;
+    list += list_entry_base(t0, I, mult);
+    uint4 *const masks = reinterpret_cast<uint4 *>(list + list_mask_base(nt, mult)), *const own_masks = masks + segment_tile(nt, w) * 32 * mult;
     const int room = (segment_tile(nt, w + 1) - segment_tile(nt, w)) * 32 * mult;
     int queued = 0, kept = 0;
     auto push = [&](T x, T y, T z, T wt, int j, unsigned ex, bool ok) {
@@ -217,7 +220,7 @@ __global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_
         queued += __popc(b);
         __syncwarp();
         if (queued >= 32) {
-            kept += test_queue<T>(S, w, lane, 32, rc2, rs2, seg + kept, room - kept, cand_pos, cand_j, cand_mask);
+            kept += test_queue<T>(S, w, lane, 32, rc2, rs2, seg + kept, room - kept, cand_pos, cand_j, own_masks + kept);
             queued -= 32;
             __syncwarp();
             if (lane < queued) {   // the rest moves to the front (read and written by the same lane)
@@ -231,10 +234,10 @@ __global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_
     // With the boxes at hand a lane looks at one of the warp's tiles each, and those whose blocks are out of range
     // as a whole (a third: the list of tiles is made for cutoff + buffer) go no further.
     for (int base = t0 + w; base < te; base += 4 * 32) {
-        const int mine = base + 4 * lane;
-        bool near_block = mine < te;
+        const int look = base + 4 * lane;
+        bool near_block = look < te;
         if (!IMAGES && boxes && near_block) {
-            const TileRec t = tiles[mine];
+            const TileRec t = tiles[look];
             const T4 bc = boxes[2 * t.J], bh = boxes[2 * t.J + 1];
             const T gx = max(T(0), abs((bc.x + (T)t.lx) + (T)t.hx - ctr[0]) - half[0] - bh.x);
             const T gy = max(T(0), abs((bc.y + (T)t.ly) + (T)t.hy - ctr[1]) - half[1] - bh.y);
@@ -308,31 +311,26 @@ __global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_
             }
         }
     }
-    if (queued) kept += test_queue<T>(S, w, lane, queued, rc2, rs2, seg + kept, room - kept, cand_pos, cand_j, cand_mask);
+    if (queued) kept += test_queue<T>(S, w, lane, queued, rc2, rs2, seg + kept, room - kept, cand_pos, cand_j, own_masks + kept);
     if (lane == 0) S.count[w] = kept;
     __syncthreads();
     if (tid == 0) ncand[I] = make_int4(S.count[0], S.count[1], S.count[2], S.count[3]);
 
     // ---- the lists, chunk by chunk
     const int e1 = S.count[0], e2 = e1 + S.count[1], e3 = e2 + S.count[2], n = e3 + S.count[3];
-    auto seg_start = [&](int q) { return ((size_t)t0 + segment_tile(nt, q)) * 32 * mult; };
-    const size_t b0 = seg_start(0), b1 = seg_start(1) - e1, b2 = seg_start(2) - e2, b3 = seg_start(3) - e3;
-    const int chunks = (n + AP_CHUNK - 1) / AP_CHUNK;
-    const int per = chunks ? (n + chunks - 1) / chunks : 0;
+    auto seg_start = [&](int q) { return segment_tile(nt, q) * 32 * mult; };
+    const int b1 = seg_start(1) - e1, b2 = seg_start(2) - e2, b3 = seg_start(3) - e3;
+    const int chunks = list_chunks(n), per = list_chunk_size(n);
     const int p = tid >> 3, s = tid & 7;
-    const size_t entries = list_entry_base(t0, I, mult), metas = list_meta_base(t0, I, mult) * 16;
+    const size_t metas = list_meta_base(t0, I, mult) * 16;
     int done = 0;   // entries of the earlier chunks
     for (int c = 0; c < chunks; ++c) {
         const int k0 = c * per, kc = min(per, n - k0);
         const int groups = (kc + 31) >> 5;
-        auto masks = [&](int g) {
-            const int k = g * 32 + lane, kk = k0 + k;
-            const size_t at = (kk < e1 ? b0 : kk < e2 ? b1 : kk < e3 ? b2 : b3) + kk;
-            return k < kc ? cand_mask[at] : make_uint4(0u, 0u, 0u, 0u);
-        };
         for (int g = w; g < groups; g += 4) {
-            const int k = g * 32 + lane;
-            const uint4 m = masks(g);
+            const int k = g * 32 + lane, kk = k0 + k;
+            uint4 m = make_uint4(0u, 0u, 0u, 0u);
+            if (k < kc) m = masks[(kk < e1 ? 0 : kk < e2 ? b1 : kk < e3 ? b2 : b3) + kk];
             unsigned in = 0u, sh = 0u, ex = 0u, own = 0u;
             if (k < kc) {
                 in = m.x;
@@ -450,14 +448,14 @@ __global__ void __launch_bounds__(LT, sizeof(T) == 4 && !IMAGES ? 8 : 5) k_pair_
             for (int k = 0; k < hole; ++k)
                 if (ph + k >= all_over) put(mine + k, s, (unsigned)kc << 4);   // the phantom
         };
-        emit(staged ? S.stage + off : list + entries + done + off);
+        emit(staged ? S.stage + off : list + done + off);
         if (s == 0)   // where it lies; its rounds of 16 entries, those with flagged and with short-range ones
             meta[metas + (size_t)c * 16 + p] = make_uint2((unsigned)(done + off), (unsigned)rounds |
                                                           ((unsigned)((r0 + 1) >> 1) << 10) | ((unsigned)((r1 + 1) >> 1) << 20));
         __syncthreads();
         if (staged) {
             const uint4 *src = reinterpret_cast<const uint4 *>(S.stage);
-            uint4 *dst = reinterpret_cast<uint4 *>(list + entries + done);
+            uint4 *dst = reinterpret_cast<uint4 *>(list + done);
             for (int k = tid; k < all / 8; k += LT) dst[k] = src[k];
         }
         done += all;
@@ -484,7 +482,7 @@ int lists_t(ap_ctx *ctx, cudaStream_t s) {
     kern<<<ctx->n_blocks, LT, sizeof(ListSmem<T>), s>>>(ctx->tiles, ctx->tile_off, ctx->excl_mask, (const T4 *)ctx->posw, boxes,
                                                         ctx->n, rc2, rs2, (T)P.box[0], (T)P.box[1], (T)P.box[2],
                                                         ctx->image_dims, ctx->list_mult, ctx->ncand, (T4 *)ctx->cand_pos,
-                                                        ctx->cand_j, ctx->cand_mask, ctx->list_meta,
+                                                        ctx->cand_j, ctx->list_meta,
                                                         (unsigned short *)ctx->list);
     AP_CUDA(cudaGetLastError());
     return AP_OK;
@@ -507,24 +505,24 @@ int lists_launch(ap_ctx *ctx, cudaStream_t s) {
 
 // (re)allocate the candidate and list arrays after a list build. The capacities hold whatever the
 // positions do: every atom of every tile a candidate, and every candidate in every target pair's
-// list (times the images an atom can have beside one block in a short box).
+// list (times the images an atom can have beside one block in a short box), an eighth more for the next
+// builds. In FP32 a tile takes 1,702 bytes: 0.52 GB at 96,000 atoms of water with r_c = 7 A and a buffer of 2 A, 5.7 GB at 1,065,000.
 int lists_alloc(ap_ctx *ctx) {
-    const long need = (long)ctx->cap_tiles * ctx->list_mult;
+    const long need = (long)ctx->n_tiles * ctx->list_mult;
     if (need <= ctx->cap_lists) return AP_OK;
-    void **ptrs[] = {(void **)&ctx->cand_j, &ctx->cand_pos, (void **)&ctx->cand_mask, (void **)&ctx->list,
+    void **ptrs[] = {(void **)&ctx->cand_j, &ctx->cand_pos, (void **)&ctx->list,
                      (void **)&ctx->list_meta};
     for (void **p : ptrs) {
         if (*p) cudaFree(*p);
         *p = nullptr;
     }
     ctx->cap_lists = 0;
-    const size_t cap = (size_t)need, es = ctx->prec == AP_FP64 ? 8 : 4;
+    const size_t cap = (size_t)(need + need / 8 + 64), es = ctx->prec == AP_FP64 ? 8 : 4;
     AP_CUDA(cudaMalloc((void **)&ctx->cand_j, sizeof(int) * 32 * cap));
     AP_CUDA(cudaMalloc(&ctx->cand_pos, 4 * es * 32 * cap));
-    AP_CUDA(cudaMalloc((void **)&ctx->cand_mask, sizeof(uint4) * 32 * cap));
     AP_CUDA(cudaMalloc((void **)&ctx->list, 2 * (AP_LIST_PER_TILE * cap + AP_LIST_PER_BLOCK * (size_t)ctx->n_blocks)));
     AP_CUDA(cudaMalloc((void **)&ctx->list_meta, sizeof(uint2) * 16 * (cap / (AP_CHUNK / 32) + ctx->n_blocks + 1)));
     if (!ctx->ncand) AP_CUDA(cudaMalloc((void **)&ctx->ncand, sizeof(int4) * ctx->n_blocks));
-    ctx->cap_lists = need;
+    ctx->cap_lists = (long)cap;
     return AP_OK;
 }

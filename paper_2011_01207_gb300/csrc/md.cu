@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(128) k_lj_forces(ListArgs la, const typename V
         sgi[h] = s0 + h < n ? (T)lj[2 * perm[s0 + h] + 1] : T(1);
     }
     double e_sum = 0.0, fi[W][3] = {};
-    const int t0 = la.tile_off[ly.I], chunks = cs.chunks(), per = chunks ? (cs.n + chunks - 1) / chunks : 0;
+    const int t0 = la.tile_off[ly.I], chunks = list_chunks(cs.n), per = list_chunk_size(cs.n);
     const unsigned *list = la.list + list_entry_base(t0, ly.I, la.mult) / 2;
     const uint2 *meta = la.meta + list_meta_base(t0, ly.I, la.mult) * 16 + ly.p;
     const T4 *cpos = (const T4 *)la.cand_pos;

@@ -47,18 +47,6 @@ inline ListArgs list_args(const ap_ctx *ctx) {
     return a;
 }
 
-// where the lists of block I start (capacities per tile and block, see lists_alloc)
-__host__ __device__ __forceinline__ size_t list_entry_base(int tile0, int I, int mult) {
-    return (size_t)tile0 * mult * AP_LIST_PER_TILE + (size_t)I * AP_LIST_PER_BLOCK;
-}
-__host__ __device__ __forceinline__ size_t list_meta_base(int tile0, int I, int mult) {
-    return ((size_t)tile0 * mult) / (AP_CHUNK / 32) + I;
-}
-
-// Warp w of the list kernel takes every fourth of a block's nt tiles, from tile w on: the first tile of its
-// segment when the warps' tiles are laid one warp after the other
-__host__ __device__ __forceinline__ int segment_tile(int nt, int w) { return w * (nt >> 2) + (w < (nt & 3) ? w : nt & 3); }
-
 // the candidates of one block: four segments (one per warp of the list kernel)
 struct Cands {
     size_t start[4];
@@ -80,7 +68,6 @@ struct Cands {
         if (k < p3) return start[2] + (k - p2);
         return start[3] + (k - p3);
     }
-    __device__ __forceinline__ int chunks() const { return (n + AP_CHUNK - 1) / AP_CHUNK; }
 };
 
 // Which block, target pair and list words a thread of a CTA of 128 has. PARTS = 1: one CTA per
@@ -297,7 +284,7 @@ __device__ __forceinline__ void for_chunks(unsigned char *raw, const ListArgs &l
                                            const typename V4<T>::type *const (&src)[NS], Body body) {
     typedef typename V4<T>::type T4;
     const Cands cs(la, ly.I);
-    const int t0 = la.tile_off[ly.I], chunks = cs.chunks(), per = chunks ? (cs.n + chunks - 1) / chunks : 0;
+    const int t0 = la.tile_off[ly.I], chunks = list_chunks(cs.n), per = list_chunk_size(cs.n);
     const unsigned *list = la.list + list_entry_base(t0, ly.I, la.mult) / 2;
     const uint2 *meta = la.meta + list_meta_base(t0, ly.I, la.mult) * 16 + ly.p;
     for (int c = 0; c < chunks; ++c) {

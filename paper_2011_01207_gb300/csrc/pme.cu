@@ -15,7 +15,6 @@
 // Grid layout: [z][y][x], x contiguous; complex half grid [z][y][x/2+1].
 #include "common.cuh"
 #include "pair_math.cuh"   // packed fma2
-#include "rules.h"
 
 #include <algorithm>
 #include <climits>
