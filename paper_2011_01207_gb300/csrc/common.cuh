@@ -235,7 +235,7 @@ int pme_multipole_field(ap_ctx *ctx, cudaStream_t s);              // permanent:
 // T_rec p -> rec; grid_cleared: the caller has zeroed the context's grid (no clearing here)
 int pme_dipole_field(ap_ctx *ctx, const void *p, cudaStream_t s, bool grid_cleared = false);
 int dipole_operator_into(ap_ctx *ctx, cudaStream_t main, cudaStream_t aux);   // T p, both branches
-// a set of PME work grids and cuFFT plans (the context owns one; others allow concurrent passes)
+// a set of PME work grids and (where the transforms are cuFFT's) plans; the context owns one, others allow concurrent passes
 struct PmeBufs {
     void *grid = nullptr, *cgrid = nullptr;
     long long *grid_fx = nullptr;

@@ -720,6 +720,15 @@ std::vector<double> moduli(int K, int order) {
     return b;
 }
 
+// cuFFT's plans of the context's sizes, where its transforms are cuFFT's
+int plans_create(ap_ctx *ctx, cufftHandle *r2c, cufftHandle *c2r) {
+    if (ctx->fft_green) return AP_OK;
+    const bool dbl = ctx->prec == AP_FP64;
+    AP_CUFFT(cufftPlan3d(r2c, ctx->K[2], ctx->K[1], ctx->K[0], dbl ? CUFFT_D2Z : CUFFT_R2C));
+    AP_CUFFT(cufftPlan3d(c2r, ctx->K[2], ctx->K[1], ctx->K[0], dbl ? CUFFT_Z2D : CUFFT_C2R));
+    return AP_OK;
+}
+
 template <class T>
 int init_t(ap_ctx *ctx) {
     const int Kx = ctx->K[0], Ky = ctx->K[1], Kz = ctx->K[2];
@@ -745,7 +754,6 @@ int init_t(ap_ctx *ctx) {
         }
     }
     AP_CUDA(cudaMemcpy(ctx->green, g.data(), sizeof(T) * g.size(), cudaMemcpyHostToDevice));
-    bool dbl = sizeof(T) == 8;
     if constexpr (std::is_same<T, float>::value) {
         AP_CUDA(cudaFuncSetAttribute(k_spread_box, cudaFuncAttributePreferredSharedMemoryCarveout, BOX_CARVEOUT));
         if (fft_supported(ctx)) {
@@ -753,8 +761,8 @@ int init_t(ap_ctx *ctx) {
             if (r) return r;
         }
     }
-    AP_CUFFT(cufftPlan3d(&ctx->plan_r2c, Kz, Ky, Kx, dbl ? CUFFT_D2Z : CUFFT_R2C));
-    AP_CUFFT(cufftPlan3d(&ctx->plan_c2r, Kz, Ky, Kx, dbl ? CUFFT_Z2D : CUFFT_C2R));
+    const int r = plans_create(ctx, &ctx->plan_r2c, &ctx->plan_c2r);
+    if (r) return r;
     if (ctx->fixed) {
         AP_CUDA(cudaMalloc((void **)&ctx->grid_fx, sizeof(long long) * ctx->ngrid));
         AP_CUDA(cudaMemset(ctx->grid_fx, 0, sizeof(long long) * ctx->ngrid));
@@ -982,12 +990,12 @@ int forces_t(ap_ctx *ctx, const void *mu4, double *gbuf, int with_M, cudaStream_
         // the transforms of the dipoles' grid and of the permanent potential, the structure-factor
         // sum over them, then the rest of the round trip
         const bool dbl = sizeof(T) == 8, own = ctx->fft_green != nullptr;
-        AP_CUFFT(cufftSetStream(bf.r2c, s));
-        AP_CUFFT(cufftSetStream(bf.c2r, s));
         if (own) {
             if ((r = fft_there_own(ctx, (const float *)ctx->grid, (float2 *)ctx->cgrid, s))) return r;
             if (with_M && (r = fft_there_own(ctx, (const float *)ctx->grid2, (float2 *)ctx->cgrid_v, s))) return r;
         } else {
+            AP_CUFFT(cufftSetStream(bf.r2c, s));
+            AP_CUFFT(cufftSetStream(bf.c2r, s));
             if (dbl) AP_CUFFT(cufftExecD2Z(bf.r2c, (cufftDoubleReal *)ctx->grid, (cufftDoubleComplex *)ctx->cgrid));
             else AP_CUFFT(cufftExecR2C(bf.r2c, (cufftReal *)ctx->grid, (cufftComplex *)ctx->cgrid));
             if (with_M) {
@@ -1078,7 +1086,7 @@ int pme_dipole_field_into(ap_ctx *ctx, const void *p, void *rec_out, const PmeBu
                                 : dipole_field_t<float>(ctx, p, rec_out, bf, s, false);
 }
 
-// a second set of grids and cuFFT plans of the context's sizes (for concurrent passes)
+// a second set of grids (and of cuFFT plans, where they are used) of the context's sizes, for concurrent passes
 int pme_bufs_create(ap_ctx *ctx, PmeBufs *b) {
     const bool dbl = ctx->prec == AP_FP64;
     const size_t es = dbl ? sizeof(double) : sizeof(float);
@@ -1088,9 +1096,7 @@ int pme_bufs_create(ap_ctx *ctx, PmeBufs *b) {
         AP_CUDA(cudaMalloc((void **)&b->grid_fx, sizeof(long long) * ctx->ngrid));
         AP_CUDA(cudaMemset(b->grid_fx, 0, sizeof(long long) * ctx->ngrid));
     }
-    AP_CUFFT(cufftPlan3d(&b->r2c, ctx->K[2], ctx->K[1], ctx->K[0], dbl ? CUFFT_D2Z : CUFFT_R2C));
-    AP_CUFFT(cufftPlan3d(&b->c2r, ctx->K[2], ctx->K[1], ctx->K[0], dbl ? CUFFT_Z2D : CUFFT_C2R));
-    return AP_OK;
+    return plans_create(ctx, &b->r2c, &b->c2r);
 }
 
 void pme_bufs_destroy(PmeBufs *b) {
