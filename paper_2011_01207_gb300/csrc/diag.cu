@@ -34,13 +34,16 @@ __global__ void __launch_bounds__(PK_THREADS) k_fma_peak(int iters, float a, flo
     if (s < -1.0f) sink[0] = s;
 }
 
-// erfc(x) as the pair kernels form it (erfc_e2 with e^{-x^2} from the same fast exponential
-// as the screened-function recursion) and CUDA's erfcf, for x >= 0
+// erfc(x) as the pair kernels form it (their screening() at beta = 1) and CUDA's erfcf, for x >= 0
 __global__ void k_erfc_pair(const float *__restrict__ x, int n, float *__restrict__ approx, float *__restrict__ lib) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float v = x[i];
-    approx[i] = erfc_e2(v, ap_fexp(-v * v));
+    PairConsts<float> pc = {};
+    pc.beta = 1.f;
+    float2 g, poly;
+    screening(RadialConsts<float>(pc), splat2(v * v), splat2(v), splat2(0.f), g, poly);
+    approx[i] = -poly.x * g.x;
     lib[i] = erfcf(v);
 }
 

@@ -15,25 +15,13 @@
 
 #include "common.cuh"
 
-__device__ __forceinline__ float ap_rsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double ap_rsqrt(double x) { return rsqrt(x); }
-__device__ __forceinline__ float ap_fexp(float x) { return __expf(x); }
-__device__ __forceinline__ double ap_fexp(double x) { return exp(x); }
-
-// erfc(x) given e2 = exp(-x^2), x >= 0. FP32: e^{-x^2} times a polynomial of degree six in
+// erfc(x), x >= 0, in FP32: e^{-x^2} times a polynomial of degree six in
 // t = 1 / (1 + 0.4 x) without constant term, the form of Abramowitz & Stegun 7.1.26 one degree
 // higher; the coefficients are a minimax fit (linear programming on 900 points of [0, 5], absolute
 // error weighted as erfc's) made for this file. In FP32 it stays within 2.0e-7 of erfc (rms 2.7e-8 on
 // [0, 4.5]; 7.1.26: 3.2e-7, 8.0e-8). FP64: the library erfc.
 #define AP_ERFC_P 0.4f
 __device__ constexpr float ERFC_C[6] = {0.232319036f, 0.159588671f, 0.473249716f, -0.376376784f, 0.712111243f, -0.200891881f};
-__device__ __forceinline__ float erfc_e2(float x, float e2) {
-    const float t = __fdividef(1.0f, fmaf(AP_ERFC_P, x, 1.0f));
-    float h = ERFC_C[5];
-#pragma unroll
-    for (int k = 4; k >= 0; --k) h = fmaf(h, t, ERFC_C[k]);
-    return h * t * e2;
-}
 
 // ---- the targets' vectors ----------------------------------------------------------------
 template <class T> struct Vec;
@@ -143,6 +131,16 @@ template <> struct RadialConsts<double> {
     __device__ __forceinline__ explicit RadialConsts(const PairConsts<double> &p) : pc(p), ta(p.thole_a) {}
 };
 
+// g = e^{-beta^2 r^2} (zero where pen says so) and poly = -erfc(beta r) / g, from r^2 and r
+__device__ __forceinline__ void screening(const RadialConsts<float> &k, float2 r2, float2 r, float2 pen, float2 &g, float2 &poly) {
+    g = ex2_2(fma2(r2, k.ce, pen));
+    const float2 t = rcp2(fma2(k.pb, r, splat2(1.0f)));
+    poly = splat2(-ERFC_C[5]);
+#pragma unroll
+    for (int n = 4; n >= 0; --n) poly = fma2(poly, t, splat2(-ERFC_C[n]));
+    poly = mul2(poly, t);
+}
+
 // -R_1..-R_N from r^2 and the Thole products tw = a w_target w_source:
 //   Mu[n] with sigma = 1, and with EX also Md[n] with sigma = 0 where exa, exb say so.
 // pen is 0 for a pair that counts and AP_OUT for one that does not (out of range): added to both
@@ -157,12 +155,8 @@ __device__ __forceinline__ void radial(const RadialConsts<float> &k, float2 r2, 
                                        float2 *Mu, float2 *Md) {
     const float2 rinv = rsqrt2(r2);
     const float2 r = mul2(r2, rinv), rinv2 = mul2(rinv, rinv);
-    const float2 g = ex2_2(fma2(r2, k.ce, pen));
-    const float2 t = rcp2(fma2(k.pb, r, splat2(1.0f)));
-    float2 poly = splat2(-ERFC_C[5]);
-#pragma unroll
-    for (int n = 4; n >= 0; --n) poly = fma2(poly, t, splat2(-ERFC_C[n]));
-    poly = mul2(poly, t);
+    float2 g, poly;
+    screening(k, r2, r, pen, g, poly);
     const float2 b1 = mul2(g, mul2(fma2(poly, rinv, k.c[0]), rinv2));   // -B_1
     const float2 s = mul2(mul2(r2, r), tw);
     const float2 e = ex2_2(fma2(s, k.nl2e, pen));
