@@ -284,14 +284,37 @@ def pairs_within(xyz, box, rc):
     return len(cKDTree(w, boxsize=box).query_pairs(rc, output_type="ndarray"))
 
 
-def launches_per_step(iters, n, rebuild_frac, guess_launches):
+def _radix_pair(k):
+    """Whether k is a product of two of the library's register transforms (2-10, 12, 14-16 points)."""
+    ok = lambda r: 2 <= r <= 10 or r == 12 or 14 <= r <= 16  # noqa: E731
+    return any(k % a == 0 and ok(a) and ok(k // a) for a in range(2, k // 2 + 1))
+
+
+def own_transforms(grid):
+    """Whether the FP32 modes' transforms on this grid are the library's three kernels (else cuFFT and a
+    product kernel): at most 96^3 points, sizes of two register transforms, and a half plane with a few
+    row pairs beside it in 227 KB of shared memory (fft.cu)."""
+    kx, ky, kz = grid
+    hx, pairs = kx // 2 + 1, (ky + 1) // 2
+    plane = lambda p: 8 * (ky * hx + p * (kx | 1) + kx + ky) + 4 * hx  # noqa: E731
+    while pairs > 4 and plane(pairs) > 227 * 1024:
+        pairs = (pairs + 1) // 2
+    return kx * ky * kz <= 96 ** 3 and all(_radix_pair(k) for k in grid) and plane(pairs) <= 227 * 1024
+
+
+def launches_per_step(iters, n, rebuild_frac, guess_launches, grid=None, sm_count=152):
     """Kernels of this library launched by one step (cuFFT's own kernels not counted)."""
+    trip = 3 if grid is not None and own_transforms(grid) else 1   # own transforms, or the product between cuFFT's
     pad = 1 if n % 32 else 0
-    field = 7 + pad                       # load, pair lists, [pad]; spread, convolve, gather, pair field,
-    #                                       assemble
+    boxes = 1 if (n + 31) // 32 >= 8 * sm_count else 0
+    field = 6 + pad + boxes + trip        # load, [pad], [block boxes], pair lists; spread, transforms, gather, pair
+    #                                       field, assemble
     guess = guess_launches
-    solve = 1 + 4 + 1 + 1 + 7 * iters + 1  # guess, matvec(4), residual (+ state), cond, 7/iter, unsort
-    forces = 10
+    one = (n + 31) // 32 * 32 <= 16384    # an iteration's vector work is one kernel, and the first direction another
+    per_iteration = 3 + trip + (1 if one else 3)   # spread, transforms, gather, pairs; vectors
+    solve = 1 + (3 + trip) + 1 + one + 1 + per_iteration * iters + 1   # guess, product, residual (+ state),
+    #                                       [direction], condition, iterations, unsort
+    forces = 9 + trip
     build = 14 * rebuild_frac
     return field + guess + solve + forces + build
 
@@ -572,7 +595,7 @@ def run_ours(args):
     it_mean = float(np.mean(iters))
     kern = {k: binding.ap_time_kernel(ctx.ctx, k, 30) for k in
             ("real_matvec", "spread_dipoles", "gather_field", "convolve", "real_field", "spread_multipoles",
-             "pair_forces")}
+             "pair_forces") if k != "convolve" or not own_transforms(grid)}
     kern["pcg_vectors"] = binding.ap_time_kernel(ctx.ctx, "pcg_vectors", 30)
     # one application of T as inside the solve (both branches), its reciprocal branch alone
     # and that branch's transforms: what bounds an iteration beside the vector kernels
@@ -683,7 +706,8 @@ def run_ours(args):
         "config": config, **cmp,
         "e2e": {"value": round(e2e_ms, 4), "unit": "ms/step", "h2d_bytes_per_step": int(s.n * 3 * 8),
                 "d2h_bytes_per_step": int(s.n * 3 * 8 + 8)},
-        "gpu_launches": int(round(launches_per_step(it_mean, s.n, 1.0 / REBUILD, launches) * args.steps)),
+        "gpu_launches": int(round(launches_per_step(it_mean, s.n, 1.0 / REBUILD, launches, grid,
+                                                    sm_count) * args.steps)),
         "kernel_ms": {k: round(v, 4) for k, v in kern.items()},
         "kernel_ms_per_step": {k: round(v, 4) for k, v in per_step.items()},
         "roofline": roofline,

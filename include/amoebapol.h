@@ -247,7 +247,8 @@ int ap_solve_info_last(ap_ctx* ctx, ap_solve_info* h_info);
 #define AP_KERNEL_REAL_MATVEC       0   /* a5: real-space dipole-field pair kernel */
 #define AP_KERNEL_REAL_FIELD        1   /* a2: real-space permanent-field pair kernel */
 #define AP_KERNEL_SPREAD_DIPOLES    2   /* a6: B-spline spread of dipoles onto the grid */
-#define AP_KERNEL_CONVOLVE          3   /* a3/a6: k-space product with B(m)C(m) */
+#define AP_KERNEL_CONVOLVE          3   /* a3/a6: k-space product with B(m)C(m) between cuFFT's transforms (part
+                                           of the transforms where they are the library's own) */
 #define AP_KERNEL_GATHER_FIELD      4   /* a3/a6: B-spline gather of the field */
 #define AP_KERNEL_SPREAD_MULTIPOLES 5   /* a3: spread of the permanent multipoles */
 #define AP_KERNEL_PAIR_FORCES       6   /* a9: real-space polarization forces and torque sources,
