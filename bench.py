@@ -702,7 +702,7 @@ def run_ours(args):
     result = {
         "metric": METRIC, "value": round(ms, 4), "unit": "ms/step", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms, 4), "higher_is_better": False, "scaling": "weak",
-        "vs_baseline": None, "dtype": "f32 pair/PME arithmetic, f64 accumulation", "data": "synthetic",
+        "vs_baseline": None, "dtype": "f32 pair/PME arithmetic, compensated f32 and f64 sums", "data": "synthetic",
         "config": config, **cmp,
         "e2e": {"value": round(e2e_ms, 4), "unit": "ms/step", "h2d_bytes_per_step": int(s.n * 3 * 8),
                 "d2h_bytes_per_step": int(s.n * 3 * 8 + 8)},
@@ -857,7 +857,7 @@ def run_replicas(args):
     print(json.dumps({
         "metric": METRIC, "value": round(ms_hist, 4), "unit": "ms per batch step (64 replicas)", "n_gpus": 1,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": round(ms_hist, 4), "higher_is_better": False,
-        "scaling": "weak", "vs_baseline": None, "dtype": "f32 pair/PME arithmetic, f64 accumulation",
+        "scaling": "weak", "vs_baseline": None, "dtype": "f32 pair/PME arithmetic, compensated f32 and f64 sums",
         "data": "synthetic",
         "config": {"workload": "replicas_64_water_and_chain_sizes_648-24000_mixed_learned_pcg1e-5",
                    "replicas": len(reps), "atoms_total": atoms, "sizes": [int(s.n) for s, _ in reps],
@@ -1327,7 +1327,7 @@ def run_two_sets(args):
     print(json.dumps({
         "metric": "two-set (d/p) polarization step ms, lockstep PCG at 1e-5 D", "impl": "ours",
         "value": round(ms2, 4), "unit": "ms/step", "steps": args.steps, "warmup": args.warmup,
-        "higher_is_better": False, "dtype": "f32 pair/PME arithmetic, f64 accumulation", "data": "synthetic",
+        "higher_is_better": False, "dtype": "f32 pair/PME arithmetic, compensated f32 and f64 sums", "data": "synthetic",
         "config": {"workload": "chain_23558_atoms_62.2A_grid64_two_sets", "atoms": s.n, "listed_pairs": int(len(pairs)),
                    "iters_mean": it2, "guess": "alpha E_d, alpha E_p",
                    "autotune": {"matvec_ctas_per_sm": tuned[0], "pme_threads": tuned[1]},

@@ -39,14 +39,17 @@ extern "C" {
 #define AP_ERR_TIMEOUT     -5   /* a bounded device wait expired */
 #define AP_ERR_STATE       -6   /* calls made out of order (e.g. solve before field) */
 
-#define AP_MIXED  0   /* FP32 pair/PME arithmetic, FP64 accumulation and PCG reductions */
+#define AP_MIXED  0   /* FP32 pair/PME arithmetic. An atom's real-space terms: FP32 sums of each thread's
+                         share of its neighbours (a few tens), compensated FP32 pairs over the threads,
+                         kept as FP64; energy, forces and virial summed over their parts in FP64, the PCG
+                         reductions in compensated pairs and FP64 */
 #define AP_FP64   1   /* FP64 everywhere (reference-grade, slow on GB300) */
 #define AP_FIXED  2   /* FP32 pair/PME arithmetic as AP_MIXED, but the PME grid and every sum that
                          several threads add to in no fixed order are accumulated in 64-bit fixed
                          point (34 fractional bits; the energy 30), as the paper's fixed-point mode
                          (Sec. 2.4); the real-space sums of an atom are one thread group's, in a
-                         fixed order, and stored in fixed point. So every output is bitwise
-                         reproducible from run to run and for any launch shape. Magnitudes must
+                         fixed order (as in AP_MIXED), and stored in fixed point. So every output is
+                         bitwise reproducible from run to run and for any launch shape. Magnitudes must
                          stay below 2^29 in the units of the output (kcal/mol/A, e/A^2). */
 
 #define AP_FRAME_NONE      0   /* multipoles given in the global frame */

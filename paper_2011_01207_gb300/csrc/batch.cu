@@ -31,9 +31,11 @@ struct ap_batch {
 namespace {
 
 // From so many replicas on, each one's kernels are captured as a single chain, without the fork and
-// join of its reciprocal branch: the replicas fill the GPU beside one another, and what the graph
-// then costs is its nodes and their cross dependencies (16 water boxes of 648 to 6,000 atoms: 4.04
-// ms a launch with the branches forked, 3.21 ms in chains).
+// join of its reciprocal branch: the replicas overlap one another, and what the graph then costs is its
+// nodes and their cross dependencies. Forked branches -> chains, ms a launch of water boxes: 4 x 648 atoms 0.80 ->
+// 0.53, 4 x 12,000 1.27 -> 1.02, 4 x 24,000 1.80 -> 1.52, 4 x 48,000 3.02 -> 2.75, 4 x 96,000 4.86 -> 4.68, 8 x 24,000 3.15 ->
+// 2.69, 16 of 648 to 6,000 3.08 -> 1.77, 16 x 24,000 6.32 -> 5.36, 64 of 648 to 24,000 17.1 -> 13.5. (Four large ones fill
+// the GPU with their pair kernels, whose neighbours' reciprocal branches run beside them either way.)
 constexpr size_t ONE_STREAM = 4;
 
 int capture_one(ap_ctx *c, const ap_batch_step &st) {

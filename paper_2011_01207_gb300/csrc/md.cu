@@ -10,10 +10,10 @@
 //     features, Sec. 2.6; 1 for constant energy); one thread per molecule, FP64 (a few
 //     hundred flops per molecule and step);
 //   * ap_lj_forces: a Lennard-Jones term, force-shifted at the real-space cutoff (energy and
-//     force continuous there), over the current configuration's in-range pair bits (each
-//     pair once) with the exclusions removed: one warp per work item, the j side through
-//     shared memory, FP64 atomics. The polarization energy is attractive, so a liquid under
-//     it alone collapses; this term supplies the repulsion of a van der Waals potential.
+//     force continuous there), over the current configuration's pair lists with the exclusions
+//     removed, each pair on the side whose source has the higher slot: one CTA per block, FP64
+//     atomics. The polarization energy is attractive, so a liquid under it alone collapses; this
+//     term supplies the repulsion of a van der Waals potential.
 // Units: A, fs, amu, kcal/mol; 1 kcal/mol/A on 1 amu accelerates by 4.184e-4 A/fs^2.
 #include "common.cuh"
 #include "pair_math.cuh"
