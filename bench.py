@@ -14,7 +14,7 @@ with the learned guess alone, the plain guess alpha E, the classical hold and th
 classical adaptive predictor (alpha E in place of the network), other guesses, the
 Jacobi/DIIS solver and the fixed-point mode are timed alongside. Inputs (every step's
 positions) are resident on the device before timing; the L2 is flushed between timed
-steps (the working set, ~60 MB, fits the 129 MB L2). `--impl reference` times the FP64
+steps (the working set, ~0.1 GB, fits the 129 MB L2). `--impl reference` times the FP64
 oracle on the host cores, full steps of the same workload. Other workloads:
 `--workload chain23k | water1m | two_sets | replicas64 | precision | kernels`.
 

@@ -84,11 +84,10 @@ __device__ __forceinline__ void block_add9(V *v, double *acc) {
 // and then
 //   F_c / f = q E_c + sum_a d_a E_ac + (1/3) sum_ab Q_ab E_abc + sum_a mu_a G_ac
 //   dU/dd / (-f) = E,   dU/dQ / (-f/3) = E_ab without its trace part (Q is traceless).
-// Measured on GB300 (ncu, warm): 228 -> 134.7 us at 96,000 atoms, 44.2 -> 23.5 us at 6,000, against
-// contracting both atoms' multipoles per pair side on 32 x 32 pair masks. 159 registers, so 3 CTAs
+// Measured on GB300 (ncu, warm): 228 -> 132.2 us at 96,000 atoms, 44.2 -> 23.5 us at 6,000, against
+// contracting both atoms' multipoles per pair side on 32 x 32 pair masks. 158 registers, so 3 CTAs
 // per SM (shared memory would hold 4): what bounds it is issue at that occupancy.
-// (Timed with events, of the 136.1 us at 96,000 atoms the compensated sums of a target's threads take 2.5 and the
-// compensated contraction 1.5.)
+// (Timed with events 135.0 us, 131.7 with the sums of a target's threads and their contraction in plain FP32.)
 // Every term is linear in the R_n, which come negated, so the sums are those of -E and -G.
 // Excluded pairs (sigma = 0 between permanent and induced, 1 between induced and induced) come
 // first in the lists and take two sets of radial functions.

@@ -26,7 +26,8 @@
 // permanent_field alone above 200,000 atoms, where nothing hides it: 693 -> 724 us at 255,552, 1,613 -> 1,752 at 648,000,
 // 2,700 -> 2,936 at 1,065,000. Interleaved tiles, entries written without a search for bits, a look at whole blocks
 // first, and two tiles in flight instead of four (64 registers, 8 CTAs an SM instead of 5: it is bound by issue and
-// latency together, 55 % of the slots at 5) made those 605, 1,443 and 2,431.
+// latency together, 55 % of the slots at 5, 68 % at 8) made those 605, 1,443 and 2,431: 91 us a launch at 96,000
+// atoms and 3 for the boxes.
 // Candidate and entry order follow the tile order, so the lists are the same in every run.
 #include "common.cuh"
 #include "pair_walk.cuh"

@@ -3,11 +3,12 @@
 // its target pairs (pair_walk.cuh); pair arithmetic and a thread's sums in T (FP32 in the mixed and fixed
 // modes), the sum over a target's threads compensated in FP32, stored once as FP64 (or fixed point).
 //
-// Bound by instruction issue (63 % of the slots busy in the matvec at 96,000 atoms, FMA pipe 36 %,
-// shared memory 35 %). Measured on GB300, ncu, warm caches, against the kernels on 32 x 32 pair
+// Bound by instruction issue and latency at the occupancy that registers and shared memory allow (63 % of the
+// slots busy in the matvec at 96,000 atoms, FMA pipe 36 %, shared memory 35 %; 53, 29 and 25 % with cold caches).
+// Measured on GB300, ncu, warm caches, against the kernels on 32 x 32 pair
 // masks that this replaced (one side per lane, items staged and flushed with atomics):
-//   matvec           96,000 atoms  61 -> 38.8 us (49.7 M -> 26 M warp instructions)
-//   permanent field  96,000 atoms  85 -> 61.7 us
+//   matvec           96,000 atoms  61 -> 40.0 us (49.7 M -> 26.6 M warp instructions)
+//   permanent field  96,000 atoms  85 -> 58.1 us
 //   matvec at 6,000 atoms (quarter blocks)  16.1 -> 8.6 us
 #include "common.cuh"
 #include "pair_math.cuh"
